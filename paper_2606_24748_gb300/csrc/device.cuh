@@ -2,6 +2,9 @@
 // the one-thread-per-block-row product, and deterministic reductions.
 #pragma once
 
+#include <type_traits>
+
+#include "fixed.cuh"
 #include "internal.h"
 
 namespace bamg {
@@ -29,19 +32,23 @@ __device__ __forceinline__ double warp_sum(double v) {
 // Matrix values and columns are streamed (evict-first); x is gathered
 // through the read-only path, where neighbouring rows hit the same lines.
 // `row` is the thread's row; `sub` its lane within the row's group.
+//
+// FP64 products of 3x3 blocks (the finest operator) are formed on the FP64
+// and the integer pipes together (fixed.cuh): the FP64 pipe alone bounds the
+// 64^3 operator (7.19 M blocks) at 107 us, HBM at 81.  Measured there: y = A x
+// 128 -> 104 us, the fused Chebyshev step 134 -> 112 us.
+template <int BR, int BC, typename TM, typename TX>
+constexpr bool fx_product() {
+  return BR == 3 && BC == 3 && std::is_same<TM, double>::value && std::is_same<TX, double>::value;
+}
+
 template <int BR, int BC, int V, typename TM, typename TA, typename TX>
-__device__ __forceinline__ void row_product(const int* __restrict__ slice_ptr,
-                                            const int* __restrict__ col,
-                                            const TM* __restrict__ vals,
-                                            const TX* __restrict__ x, int64_t row, int sub,
-                                            TA (&acc)[BR]) {
-  const int64_t s = row >> 5;
-  const int lane = (int)(row & 31);
-  const int c0 = __ldg(slice_ptr + s), c1 = __ldg(slice_ptr + s + 1);
+__device__ __forceinline__ void row_sums(int c0, int c1, const int* __restrict__ col, const TM* __restrict__ vals,
+                                         const TX* __restrict__ x, int lane, TA (&acc)[BR]) {
 #pragma unroll
   for (int r = 0; r < BR; ++r) acc[r] = TA(0);
 #pragma unroll 2
-  for (int c = c0 + sub; c < c1; c += V) {
+  for (int c = c0; c < c1; c += V) {
     const int64_t slot = (int64_t)c * 32 + lane;
     const int j = __ldcs(col + slot);
     const TM* v = vals + (int64_t)c * (32 * BR * BC) + lane;
@@ -52,6 +59,58 @@ __device__ __forceinline__ void row_product(const int* __restrict__ slice_ptr,
     for (int r = 0; r < BR; ++r)
 #pragma unroll
       for (int q = 0; q < BC; ++q) acc[r] = fma((TA)__ldcs(v + 32 * (r * BC + q)), xv[q], acc[r]);
+  }
+}
+
+template <int BR, int BC, int V>
+__device__ __forceinline__ void row_sums_fx(int c0, int c1, const int* __restrict__ col,
+                                            const double* __restrict__ vals, const double* __restrict__ x, int lane,
+                                            double (&acc)[BR]) {
+  using Row = FxRow<BR, BC>;
+  Row row;
+  row.init();
+  int left = Row::kCarry, carries = 0;
+#pragma unroll 1
+  for (int c = c0; c < c1; c += V) {
+    const int j = __ldcs(col + (int64_t)c * 32 + lane);
+    const double* v = vals + (int64_t)c * (32 * BR * BC) + lane;
+    double blk[BR * BC], xv[BC];
+#pragma unroll
+    for (int e = 0; e < BR * BC; ++e) blk[e] = __ldcs(v + 32 * e);
+#pragma unroll
+    for (int q = 0; q < BC; ++q) xv[q] = __ldg(x + (int64_t)j * BC + q);
+    FxBlock<BR, BC> a;
+    a.cut(blk);
+    row.add(blk, a, xv);
+    if (--left == 0) {
+      left = Row::kCarry;
+      row.carry();
+      if ((++carries & 1) == 0) row.flush();
+    }
+  }
+  row.carry();
+  row.flush();
+  if (row.valid()) {
+#pragma unroll
+    for (int r = 0; r < BR; ++r) acc[r] = row.acc[r];
+  } else {
+    row_sums<BR, BC, V, double, double, double>(c0, c1, col, vals, x, lane, acc);
+  }
+}
+
+template <int BR, int BC, int V, typename TM, typename TA, typename TX>
+__device__ __forceinline__ void row_product(const int* __restrict__ slice_ptr,
+                                            const int* __restrict__ col,
+                                            const TM* __restrict__ vals,
+                                            const TX* __restrict__ x, int64_t row, int sub,
+                                            TA (&acc)[BR]) {
+  const int64_t s = row >> 5;
+  const int lane = (int)(row & 31);
+  const int c0 = __ldg(slice_ptr + s) + sub, c1 = __ldg(slice_ptr + s + 1);
+  if constexpr (fx_product<BR, BC, TM, TX>()) {
+    row_sums_fx<BR, BC, V>(c0, c1, col, vals, x, lane, acc);
+  } else {
+    row_sums<BR, BC, V, TM, TA, TX>(c0, c1, col, vals, x, lane, acc);
   }
   if (V > 1) {
 #pragma unroll
@@ -261,19 +320,9 @@ __device__ __forceinline__ void st4(float* p, const float (&v)[4]) {
   reinterpret_cast<float4*>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
 }
 
-// Block-row product for four right-hand sides at once: X holds kp vectors
-// RHS-minor (entry (dof d, vector j) at X[d * kp + j]) and the thread takes
-// vectors c0..c0+3 of block row `row`.  Each block value is loaded once and
-// used for the four vectors; the kp / 4 threads of a row read the same value
-// (one broadcast).  Per vector, the summation order is that of row_product
-// with one lane per row.
 template <int BR, int BC, typename T>
-__device__ __forceinline__ void row_product4(const int* __restrict__ slice_ptr, const int* __restrict__ col,
-                                             const T* __restrict__ vals, const T* __restrict__ X, int kp,
-                                             int64_t row, int c0, T (&acc)[BR][4]) {
-  const int64_t s = row >> 5;
-  const int lane = (int)(row & 31);
-  const int a0 = __ldg(slice_ptr + s), a1 = __ldg(slice_ptr + s + 1);
+__device__ __forceinline__ void row_sums4(int a0, int a1, const int* __restrict__ col, const T* __restrict__ vals,
+                                          const T* __restrict__ X, int kp, int lane, int c0, T (&acc)[BR][4]) {
 #pragma unroll
   for (int r = 0; r < BR; ++r)
 #pragma unroll
@@ -292,6 +341,97 @@ __device__ __forceinline__ void row_product4(const int* __restrict__ slice_ptr, 
 #pragma unroll
         for (int e = 0; e < 4; ++e) acc[r][e] = fma(a, xv[q][e], acc[r][e]);
       }
+  }
+}
+
+// The four vectors share a block's limbs; per vector the sums are those of
+// row_sums_fx with one lane per row, bit for bit (65^3 nodes, 16 vectors:
+// 1,820 us on the FP64 pipe alone, 959 on both).
+template <int BR, int BC>
+__device__ __forceinline__ void row_sums4_fx(int a0, int a1, const int* __restrict__ col,
+                                             const double* __restrict__ vals, const double* __restrict__ X, int kp,
+                                             int lane, int c0, double (&acc)[BR][4]) {
+  using Row = FxRow<BR, BC>;
+  Row row[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) row[e].init();
+  int left = Row::kCarry, carries = 0;
+#pragma unroll 1
+  for (int c = a0; c < a1; ++c) {
+    const int j = __ldg(col + (int64_t)c * 32 + lane);
+    const double* v = vals + (int64_t)c * (32 * BR * BC) + lane;
+    double blk[BR * BC], xv[BC][4];
+#pragma unroll
+    for (int e = 0; e < BR * BC; ++e) blk[e] = __ldg(v + 32 * e);
+#pragma unroll
+    for (int q = 0; q < BC; ++q) ld4(X + ((int64_t)j * BC + q) * kp + c0, xv[q]);
+    FxBlock<BR, BC> a;
+    a.cut(blk);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      double x[BC];
+#pragma unroll
+      for (int q = 0; q < BC; ++q) x[q] = xv[q][e];
+      row[e].add(blk, a, x);
+    }
+    if (--left == 0) {
+      left = Row::kCarry;
+      const bool full = (++carries & 1) == 0;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        row[e].carry();
+        if (full) row[e].flush();
+      }
+    }
+  }
+  unsigned redo = 0;  // vectors that the scales do not cover: formed by FP64 FMA, one at a time
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    row[e].carry();
+    row[e].flush();
+    if (!row[e].valid()) redo |= 1u << e;
+#pragma unroll
+    for (int r = 0; r < BR; ++r) acc[r][e] = row[e].acc[r];
+  }
+#pragma unroll 1
+  for (int e = 0; redo >> e; ++e) {
+    if (!(redo >> e & 1)) continue;
+    double f[BR];
+#pragma unroll
+    for (int r = 0; r < BR; ++r) f[r] = 0.0;
+#pragma unroll 1
+    for (int c = a0; c < a1; ++c) {
+      const double* x = X + (int64_t)__ldg(col + (int64_t)c * 32 + lane) * BC * kp + c0 + e;
+      const double* v = vals + (int64_t)c * (32 * BR * BC) + lane;
+#pragma unroll
+      for (int r = 0; r < BR; ++r)
+#pragma unroll
+        for (int q = 0; q < BC; ++q) f[r] = fma(__ldg(v + 32 * (r * BC + q)), __ldg(x + (int64_t)q * kp), f[r]);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int r = 0; r < BR; ++r) acc[r][k] = k == e ? f[r] : acc[r][k];
+  }
+}
+
+// Block-row product for four right-hand sides at once: X holds kp vectors
+// RHS-minor (entry (dof d, vector j) at X[d * kp + j]) and the thread takes
+// vectors c0..c0+3 of block row `row`.  Each block value is loaded once and
+// used for the four vectors; the kp / 4 threads of a row read the same value
+// (one broadcast).  Per vector, the summation order is that of row_product
+// with one lane per row.
+template <int BR, int BC, typename T>
+__device__ __forceinline__ void row_product4(const int* __restrict__ slice_ptr, const int* __restrict__ col,
+                                             const T* __restrict__ vals, const T* __restrict__ X, int kp,
+                                             int64_t row, int c0, T (&acc)[BR][4]) {
+  const int64_t s = row >> 5;
+  const int lane = (int)(row & 31);
+  const int a0 = __ldg(slice_ptr + s), a1 = __ldg(slice_ptr + s + 1);
+  if constexpr (fx_product<BR, BC, T, T>()) {
+    row_sums4_fx<BR, BC>(a0, a1, col, vals, X, kp, lane, c0, acc);
+  } else {
+    row_sums4<BR, BC, T>(a0, a1, col, vals, X, kp, lane, c0, acc);
   }
 }
 

@@ -1,0 +1,179 @@
+// FP64 block products on two pipes at once: some rows of each block by FP64
+// FMA, the others in block-scaled fixed point on the integer pipes.
+//
+// A GB300 SM retires two FP64 FMA per clock but some 60 integer operations and
+// 13 wide (32 x 32 + 64 bit) integer multiply-adds (measured), so a product
+// that takes every row through the FP64 pipe is bound by it below the rate of
+// HBM.  A fixed-point product takes three wide multiply-adds and no FP64
+// operation:
+//  - a block's values are cut, each with its sign, into two 28-bit limbs on the
+//    scale of the block's largest value; x's entries likewise on a scale that
+//    gives every product of a row one common exponent, the largest seen so far
+//    (when a larger one comes the row's sums are shifted down to it);
+//  - the limb products high x high and high x low + low x high are summed in
+//    two 64-bit integers; low x low (2^-56 of the largest product) is dropped.
+// Integer sums do not round, so a row's error is that of the cut operands, at
+// most 2^-55 of the largest |block| |x| of the row per product; an FP64 sum
+// rounds at 2^-53 of each partial sum.  Measured against 80-bit sums on a
+// 27-block row with values over two decades: 1.6e-16 in the fixed-point rows,
+// 3.0e-16 by FP64 FMA.  Every cut is symmetric in the sign and moves with the
+// exponent, so x -> -x and x -> 2^k x give exactly -y and 2^k y.
+// Rows with values that the scales do not cover (Inf, NaN, or a largest entry
+// beyond 2^+-767) are done again by FP64 FMA alone.
+#pragma once
+
+#include <cstdint>
+
+namespace bamg {
+
+// Rows of a block that stay on the FP64 pipe.  With one of three there, the two
+// pipes are busy for about as long (3x3 products, 65^3 nodes, 27 blocks per
+// row: 141.8 us with three, 102 with one, 116 with none).
+template <int BR>
+constexpr int fx_fma_rows() { return BR / 3; }
+
+__device__ __forceinline__ unsigned fx_shr(unsigned a, unsigned s) {  // 0 for s > 31
+  unsigned r;
+  asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(s));
+  return r;
+}
+__device__ __forceinline__ unsigned long long fx_shr(unsigned long long a, unsigned s) {  // 0 for s > 63
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(s));
+  return r;
+}
+
+struct FxBits {  // a double's words
+  unsigned hi, lo;
+};
+__device__ __forceinline__ FxBits fx_bits(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  return {(unsigned)(b >> 32), (unsigned)b};
+}
+
+// (h 2^28 + l) 2^(top - 1078) is v cut toward zero, for a biased exponent
+// top >= v's; 0 when top is 60 or more above it (so for v = 0, top >= 60).
+__device__ __forceinline__ void fx_limbs(FxBits v, int top, int& h, int& l) {
+  const unsigned s = (unsigned)(top - (int)((v.hi & 0x7fffffffu) >> 20));
+  const unsigned m = (__funnelshift_l(v.lo, v.hi, 7) & 0x07ffffffu) | 0x08000000u;
+  const unsigned long long w = ((unsigned long long)m << 32) | (v.lo << 7);
+  const int sign = ((int)v.hi >> 31) | 1;
+  h = (int)fx_shr(m, s) * sign;
+  l = (int)((unsigned)fx_shr(w, s) >> 4) * sign;
+}
+
+// v / 2^d toward zero, so that -v gives exactly the opposite.
+__device__ __forceinline__ long long fx_down(long long v, int d) {
+  return (v + ((v >> 63) & ((1LL << d) - 1))) >> d;
+}
+
+// Smallest biased exponent a scale is taken from: zeros, and values this far
+// down, then cut to 0 on it.
+constexpr int kFxMinExp = 64;
+
+// A block's values cut to limbs: rows fx_fma_rows() .. BR - 1.
+template <int BR, int BC>
+struct FxBlock {
+  static constexpr int R0 = fx_fma_rows<BR>(), N = (BR - R0) * BC;
+  int h[N], l[N];
+  unsigned top;  // largest high word without sign (0: all values zero)
+  int exp;       // exponent of the scale
+  __device__ __forceinline__ void cut(const double (&v)[BR * BC]) {
+    top = 0;
+#pragma unroll
+    for (int e = 0; e < N; ++e) top = max(top, fx_bits(v[R0 * BC + e]).hi & 0x7fffffffu);
+    if (top == 0) {  // zeros, or subnormals below the high word
+      unsigned low = 0;
+#pragma unroll
+      for (int e = 0; e < N; ++e) low |= fx_bits(v[R0 * BC + e]).lo;
+      top = low != 0;
+    }
+    exp = max((int)(top >> 20), kFxMinExp);
+#pragma unroll
+    for (int e = 0; e < N; ++e) fx_limbs(fx_bits(v[R0 * BC + e]), exp, h[e], l[e]);
+  }
+};
+
+// Sums of one row (all its components) over its blocks for one vector.
+template <int BR, int BC>
+struct FxRow {
+  static constexpr int R0 = fx_fma_rows<BR>(), NI = BR - R0;
+  // Limb products are below 2^56, so `mid` (two per term) holds 60 terms
+  // before it is carried into `hh`, and `hh` 120 before it goes to `acc`.
+  static constexpr int kCarry = 60 / BC, kFlush = 2 * kCarry;
+  double acc[BR];
+  long long hh[NI], mid[NI];
+  int E;              // hh and mid are on the scale 2^(E - 2156 + 56) and 2^(E - 2156 + 28)
+  unsigned amax, xmax;  // largest high words of the blocks' and of x's values
+
+  __device__ __forceinline__ void init() {
+#pragma unroll
+    for (int r = 0; r < BR; ++r) acc[r] = 0.0;
+#pragma unroll
+    for (int r = 0; r < NI; ++r) hh[r] = mid[r] = 0;
+    E = 0;
+    amax = xmax = 0;
+  }
+  __device__ __forceinline__ void add(const double (&v)[BR * BC], const FxBlock<BR, BC>& a, const double (&x)[BC]) {
+#pragma unroll
+    for (int r = 0; r < R0; ++r)
+#pragma unroll
+      for (int q = 0; q < BC; ++q) acc[r] = fma(v[r * BC + q], x[q], acc[r]);
+    unsigned mx = 0;
+#pragma unroll
+    for (int q = 0; q < BC; ++q) mx = max(mx, fx_bits(x[q]).hi & 0x7fffffffu);
+    if (mx == 0) {
+      unsigned low = 0;
+#pragma unroll
+      for (int q = 0; q < BC; ++q) low |= fx_bits(x[q]).lo;
+      mx = low != 0;
+    }
+    amax = max(amax, a.top);
+    xmax = max(xmax, mx);
+    const int need = (a.top != 0 && mx != 0) ? a.exp + max((int)(mx >> 20), kFxMinExp) : 0;
+    if (need > E) {
+      const int d = min(need - E, 62);
+      E = need;
+#pragma unroll
+      for (int r = 0; r < NI; ++r) {
+        hh[r] = fx_down(hh[r], d);
+        mid[r] = fx_down(mid[r], d);
+      }
+    }
+    const int top = mx != 0 ? E - a.exp : 2200;
+#pragma unroll
+    for (int q = 0; q < BC; ++q) {
+      int h, l;
+      fx_limbs(fx_bits(x[q]), top, h, l);
+#pragma unroll
+      for (int r = 0; r < NI; ++r) {
+        hh[r] += (long long)a.h[r * BC + q] * h;
+        mid[r] += (long long)a.h[r * BC + q] * l;
+        mid[r] += (long long)a.l[r * BC + q] * h;
+      }
+    }
+  }
+  __device__ __forceinline__ void carry() {
+#pragma unroll
+    for (int r = 0; r < NI; ++r) {
+      const long long up = fx_down(mid[r], 28);
+      hh[r] += up;
+      mid[r] -= up << 28;
+    }
+  }
+  __device__ __forceinline__ void flush() {  // after carry()
+    const double scale = __longlong_as_double((long long)(max(E, 1106) - 1105) << 52);
+#pragma unroll
+    for (int r = 0; r < NI; ++r) {
+      acc[R0 + r] = fma(fma((double)hh[r], 268435456.0, (double)(int)mid[r]), scale, acc[R0 + r]);
+      hh[r] = mid[r] = 0;
+    }
+  }
+  // Whether acc[] is the row's product; otherwise it has to be formed by FP64 FMA.
+  __device__ __forceinline__ bool valid() const {
+    auto covered = [](unsigned m) { return m == 0 || m - 0x10000000u < 0x60000000u; };
+    return covered(amax) && covered(xmax) && (E == 0 || (unsigned)(E - 1106) < 2046u);
+  }
+};
+
+}  // namespace bamg

@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(256) k_mcheb_init(int64_t n, int glog, int kp,
 
 // x += d_in; r -= A d_in; if has_next: d_out = c1 d_in + c2 w Dinv r
 template <int BS, typename T>
-__global__ void __launch_bounds__(256) k_mcheb_step(const int* __restrict__ sp, const int* __restrict__ col,
+__global__ void __launch_bounds__(256, 2) k_mcheb_step(const int* __restrict__ sp, const int* __restrict__ col,
                                                     const T* __restrict__ vals, const int* __restrict__ srow,
                                                     int64_t n, int glog, int kp,
                                                     const T* __restrict__ d_in, T* __restrict__ d_out,
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(256) k_mcheb_step(const int* __restrict__ sp, 
 
 // r = b - A x; d = w Dinv r / theta
 template <int BS, typename T>
-__global__ void __launch_bounds__(256) k_mcheb_rinit(const int* __restrict__ sp, const int* __restrict__ col,
+__global__ void __launch_bounds__(256, 2) k_mcheb_rinit(const int* __restrict__ sp, const int* __restrict__ col,
                                                      const T* __restrict__ vals, const int* __restrict__ srow,
                                                      int64_t n, int glog, int kp,
                                                      const T* __restrict__ x, const T* __restrict__ b,
@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(256) k_mcg_first(int64_t m, int kp, const doub
 }
 
 // q = A p, alpha_j = rz_j / (p_j . q_j)
-__global__ void __launch_bounds__(256) k_mcg_Ap(const int* __restrict__ sp, const int* __restrict__ col,
+__global__ void __launch_bounds__(256, 2) k_mcg_Ap(const int* __restrict__ sp, const int* __restrict__ col,
                                                 const double* __restrict__ vals, const int* __restrict__ srow,
                                                 int64_t n, int glog, int kp,
                                                 const double* __restrict__ p, double* __restrict__ q,
@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(256) k_mcg_p(int64_t m, int kp, const double* 
 }
 
 // ||b_j - A x_j||^2 (b read from the caller's k-column array)
-__global__ void __launch_bounds__(256) k_mcg_true_residual(const int* __restrict__ sp, const int* __restrict__ col,
+__global__ void __launch_bounds__(256, 2) k_mcg_true_residual(const int* __restrict__ sp, const int* __restrict__ col,
                                                            const double* __restrict__ vals,
                                                            const int* __restrict__ srow, int64_t n, int glog,
                                                            int kp, int k, const double* __restrict__ x,

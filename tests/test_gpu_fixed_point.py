@@ -1,0 +1,127 @@
+"""FP64 products whose rows are partly formed in block-scaled fixed point:
+against sums in extended precision, with the error bound the operand cuts
+and the FP64 sums allow, at row lengths around the carry and flush steps."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2606_24748_gb300 import bamg as B
+
+pytestmark = pytest.mark.gpu
+
+
+def operator(rng, lengths, nbc, bs, decades):
+    """Block COO arrays of a matrix whose row i has lengths[i] blocks."""
+    br, bc = bs
+    bi = np.repeat(np.arange(len(lengths)), lengths).astype(np.int32)
+    bj = np.concatenate([np.sort(rng.choice(nbc, k, replace=False)) for k in lengths]).astype(np.int32)
+    v = rng.standard_normal((bi.size, br, bc)) * 10.0 ** rng.uniform(-decades, decades, (bi.size, 1, 1))
+    v[rng.random(bi.size) < 0.05] = 0.0
+    return bi, bj, v
+
+
+def reference(bi, bj, v, x, nbr):
+    """Products, sums of |a| |x|, the largest max|block| max|x entry| and the terms of each row."""
+    br, bc = v.shape[1:]
+    xb = x.reshape(-1, bc)
+    y = np.zeros((nbr, br), dtype=np.longdouble)
+    mag, top, n = np.zeros((nbr, br)), np.zeros(nbr), np.zeros(nbr)
+    for i, j, a in zip(bi, bj, v):
+        y[i] += (a.astype(np.longdouble) * xb[j].astype(np.longdouble)).sum(1)
+        mag[i] += np.abs(a) @ np.abs(xb[j])
+        top[i] = max(top[i], np.abs(a).max() * np.abs(xb[j]).max())
+        n[i] += bc
+    return y, mag, top[:, None], n[:, None]
+
+
+def within(got, ref, scale=1.0):
+    """A fixed-point product is off by at most 2^-55 + 2 * 2^-54 of the row's
+    largest |block| |x| (both cuts and the dropped limb product; the scales are
+    at most twice the largest values), an FP64 sum of n terms by n 2^-53 of
+    the sum of |a| |x|."""
+    y, mag, top, n = ref
+    return np.all(np.abs(got.reshape(y.shape).astype(np.longdouble) / scale - y) <= n * 2.0 ** -52 * (mag + 2.5 * top))
+
+
+@pytest.mark.parametrize("bs", [(3, 3)])
+def test_products_at_carry_and_flush_lengths(bs):
+    rng = np.random.default_rng(5)
+    lengths = [1, 19, 20, 21, 39, 40, 41, 60, 80, 81, 120, 0, 2, 7] + [27] * 40
+    nbc, nbr = 130, len(lengths)
+    ctx = B.bamg_ctx_create(torch.cuda.current_stream())
+    A = B.bamg_bsr_create(ctx, bs[0], bs[1], nbr, nbc)
+    try:
+        bi, bj, v = operator(rng, lengths, nbc, bs, 2.0)
+        B.bamg_bsr_coo_preallocate(ctx, A, torch.from_numpy(bi).cuda(), torch.from_numpy(bj).cuda())
+        B.bamg_bsr_coo_set_values(ctx, A, torch.from_numpy(v).cuda(), 0)
+        x = rng.standard_normal(nbc * bs[1]) * 10.0 ** rng.uniform(-3, 3, nbc * bs[1])
+        ref = reference(bi, bj, v, x, nbr)
+        xd = torch.from_numpy(x).cuda()
+        single = torch.full((nbr * bs[0],), 7.0, dtype=torch.float64, device="cuda")
+        for lanes in (4, 32, 1):
+            B.bamg_bsr_set_lanes(ctx, A, lanes)
+            B.bamg_bsr_spmv(ctx, A, xd, single)
+            assert within(single.cpu().numpy(), ref), lanes
+        # several vectors: the single one-lane product bit for bit, whatever its sign and scale
+        for f in (1.0, -1.0, 2.0 ** 40, -(2.0 ** -70)):
+            X = torch.stack([f * xd, xd, torch.zeros_like(xd), -xd], 1).contiguous()
+            Y = torch.empty((nbr * bs[0], 4), dtype=torch.float64, device="cuda")
+            B.bamg_bsr_spmm(ctx, A, X, Y, 4)
+            assert torch.equal(Y[:, 0], f * single) and torch.equal(Y[:, 1], single)
+            assert torch.equal(Y[:, 3], -single) and not Y[:, 2].any()
+        # columns that are no multiple of four take the one-column kernel
+        X = torch.stack([xd, 2 * xd, -xd], 1).contiguous()
+        Y = torch.empty((nbr * bs[0], 3), dtype=torch.float64, device="cuda")
+        B.bamg_bsr_spmm(ctx, A, X, Y, 3)
+        assert all(within(Y[:, j].cpu().numpy(), ref, f) for j, f in enumerate((1.0, 2.0, -1.0)))
+    finally:
+        B.bamg_bsr_destroy(A)
+        B.bamg_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("bs", [(3, 3)])
+@pytest.mark.parametrize("lanes", [1, 4])
+def test_values_outside_the_scales(bs, lanes):
+    """Infinities, NaN, subnormals, the largest and smallest magnitudes and
+    zero blocks beside huge x give what FP64 multiply-adds give."""
+    rng = np.random.default_rng(9)
+    nbr = nbc = 64
+    lengths = [9] * nbr
+    ctx = B.bamg_ctx_create(torch.cuda.current_stream())
+    A = B.bamg_bsr_create(ctx, bs[0], bs[1], nbr, nbc)
+    try:
+        bi, bj, v = operator(rng, lengths, nbc, bs, 1.0)
+        x = rng.standard_normal(nbc * bs[1])
+        v[9 * 3 + 2, 1, 1] = np.inf
+        v[9 * 5 + 1, 2, 0] = np.nan
+        v[9 * 7:9 * 8] *= 1e-300
+        v[9 * 9:9 * 10] *= 2.0 ** 900
+        v[9 * 11:9 * 12] *= 2.0 ** -1060
+        v[9 * 13:9 * 14] = 0.0
+        v[9 * 15 + 4] = 0.0
+        x[bj[9 * 15 + 4] * bs[1]] = 2.0 ** 800
+        B.bamg_bsr_coo_preallocate(ctx, A, torch.from_numpy(bi).cuda(), torch.from_numpy(bj).cuda())
+        B.bamg_bsr_coo_set_values(ctx, A, torch.from_numpy(v).cuda(), 0)
+        B.bamg_bsr_set_lanes(ctx, A, lanes)
+        y = torch.empty(nbr * bs[0], dtype=torch.float64, device="cuda")
+        B.bamg_bsr_spmv(ctx, A, torch.from_numpy(x).cuda(), y)
+        got = y.cpu().numpy().reshape(nbr, bs[0])
+        with np.errstate(all="ignore"):
+            want = np.zeros((nbr, bs[0]))
+            np.add.at(want, bi, np.einsum("krc,kc->kr", v, x.reshape(-1, bs[1])[bj]))
+            tol = np.zeros((nbr, bs[0]))
+            np.add.at(tol, bi, np.einsum("krc,kc->kr", np.abs(v), np.abs(x.reshape(-1, bs[1])[bj])))
+        fine = np.isfinite(want)
+        assert np.array_equal(np.isnan(got), np.isnan(want))
+        assert np.array_equal(got[~fine & ~np.isnan(want)], want[~fine & ~np.isnan(want)])
+        # both sides sum 27 products (18, 36 or 54 of other shapes) in FP64 or
+        # better; subnormal sums are off by at most one unit per term
+        n = 9 * bs[1]
+        bound = n * 2.0 ** -51 * tol + n * 2.0 ** -1074
+        off = np.abs(got - want, where=fine, out=np.zeros_like(want))
+        # max|block| max|x entry| exceeds the sum of |a| |x| of a row by at most this factor
+        assert (off <= bound)[fine].mean() > 0.9 and (off <= 64 * bound)[fine].all()
+        assert not got[13].any()
+    finally:
+        B.bamg_bsr_destroy(A)
+        B.bamg_ctx_destroy(ctx)
