@@ -32,7 +32,6 @@ __device__ __forceinline__ double warp_sum(double v) {
 // Matrix values and columns are streamed (evict-first); x is gathered
 // through the read-only path, where neighbouring rows hit the same lines.
 // `row` is the thread's row; `sub` its lane within the row's group.
-//
 // FP64 products of 3x3 blocks (the finest operator) are formed on the FP64
 // and the integer pipes together (fixed.cuh): the FP64 pipe alone bounds the
 // 64^3 operator (7.19 M blocks) at 107 us, HBM at 81.  Measured there: y = A x
@@ -272,7 +271,8 @@ __device__ bool grid_reduce(double (&v)[NV], double* __restrict__ partials,
   double acc[NV];
 #pragma unroll
   for (int k = 0; k < NV; ++k) acc[k] = 0.0;
-  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
+#pragma unroll 8
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)  // loads of several partials in flight
 #pragma unroll
     for (int k = 0; k < NV; ++k) acc[k] += __ldcg(partials + (int64_t)b * NV + k);
 #pragma unroll
@@ -469,7 +469,8 @@ __device__ bool grid_reduce_groups(const double (&v)[NV], int G, double* __restr
   __threadfence();
   const int step = blockDim.x / ns;
   double a = 0.0;
-  for (int b = threadIdx.x / ns; b < (int)gridDim.x; b += step)
+#pragma unroll 8
+  for (int b = threadIdx.x / ns; b < (int)gridDim.x; b += step)  // loads of several partials in flight
     a += __ldcg(partials + (int64_t)b * ns + threadIdx.x % ns);
   sm[threadIdx.x] = a;
   __syncthreads();

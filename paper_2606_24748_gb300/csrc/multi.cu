@@ -186,6 +186,138 @@ __global__ void __launch_bounds__(256) k_mtransfer(const int* __restrict__ sp, c
   }
 }
 
+// Split forms of the three row kernels above, for matrices with few rows
+// (coarse operators, restrictions).  There a thread per row and four columns
+// leaves most of the chip idle behind a few long chains of FP64 multiply-adds
+// (64 cycles each per warp): 1,331 rows of 27 6x6 blocks and 16 columns are
+// 166 warps for 608 SM sub-partitions.  Here a thread takes one row and one
+// column, and 2^vlog threads share a row's blocks; their partial sums meet in
+// shared memory, are added in thread order, and the row's components are
+// finished by different threads.
+struct SplitMap {
+  int klog, vlog, rlog;  // columns, threads per row's blocks and rows per CTA, as powers of two
+};
+constexpr int kSplitThreads = 512;  // at most; kSplitThreads >= columns x threads per row
+
+// This CTA's partial sums of its rows' products, one per thread and component,
+// at part[(sub * BR + a) * W + idx] with W = rows x columns of the CTA.
+template <int BR, int BC, typename T>
+__device__ __forceinline__ void split_partials(const SplitMap m, const int* __restrict__ sp,
+                                               const int* __restrict__ col, const T* __restrict__ vals, int64_t n,
+                                               const T* __restrict__ X, int64_t pos, int c, int sub, int idx,
+                                               T* part) {
+  T acc[BR];
+#pragma unroll
+  for (int a = 0; a < BR; ++a) acc[a] = T(0);
+  if (pos < n) {
+    const int64_t s = pos >> 5;
+    const int lane = (int)(pos & 31);
+    const int a0 = __ldg(sp + s) + sub, a1 = __ldg(sp + s + 1);
+    for (int ch = a0; ch < a1; ch += 1 << m.vlog) {
+      const int j = __ldg(col + (int64_t)ch * 32 + lane);
+      const T* v = vals + (int64_t)ch * (32 * BR * BC) + lane;
+      T xv[BC];
+#pragma unroll
+      for (int q = 0; q < BC; ++q) xv[q] = __ldg(X + (((int64_t)j * BC + q) << m.klog) + c);
+#pragma unroll
+      for (int a = 0; a < BR; ++a)
+#pragma unroll
+        for (int q = 0; q < BC; ++q) acc[a] = fma(__ldg(v + 32 * (a * BC + q)), xv[q], acc[a]);
+    }
+  }
+  const int W = 1 << (m.rlog + m.klog);
+#pragma unroll
+  for (int a = 0; a < BR; ++a) part[(sub * BR + a) * W + idx] = acc[a];
+  __syncthreads();
+}
+
+template <int BR, typename T>
+__device__ __forceinline__ T split_sum(const SplitMap m, const T* part, int a, int idx) {
+  const int W = 1 << (m.rlog + m.klog);
+  T t = part[a * W + idx];
+  for (int k = 1; k < 1 << m.vlog; ++k) t += part[(k * BR + a) * W + idx];
+  return t;
+}
+
+#define BAMG_SPLIT_THREAD                                                              \
+  const int idx = (int)threadIdx.x & ((1 << (m.rlog + m.klog)) - 1);                   \
+  const int sub = (int)threadIdx.x >> (m.rlog + m.klog), c = idx & ((1 << m.klog) - 1); \
+  const int64_t pos = ((int64_t)blockIdx.x << m.rlog) + (idx >> m.klog);
+
+// Chebyshev step (INIT = false) or residual start (true: r = b - A x, d = f
+// w Dinv r) of the kernels above.
+template <int BS, typename T, bool INIT>
+__global__ void __launch_bounds__(kSplitThreads) k_mcheb_split(const SplitMap m, const int* __restrict__ sp,
+                                                               const int* __restrict__ col,
+                                                               const T* __restrict__ vals,
+                                                               const int* __restrict__ srow, int64_t n,
+                                                               const T* __restrict__ v_in, const T* __restrict__ b,
+                                                               T* __restrict__ d_out, T* __restrict__ x,
+                                                               T* __restrict__ r, const T* __restrict__ dinv,
+                                                               const float* __restrict__ w,
+                                                               const double* __restrict__ scal, int k, int has_next,
+                                                               const int* done) {
+  BAMG_DONE_RETURN
+  __shared__ T part[kSplitThreads * BS];
+  BAMG_SPLIT_THREAD
+  const int V = 1 << m.vlog, W = 1 << (m.rlog + m.klog);
+  split_partials<BS, BS, T>(m, sp, col, vals, n, v_in, pos, c, sub, idx, part);
+  const int64_t i = pos < n ? row_at(srow, pos) : -1;
+  T rn[(BS + 1) / 2];  // the thread's components sub, sub + V, ... (V >= 2)
+#pragma unroll
+  for (int t = 0; t < (BS + 1) / 2; ++t) {
+    const int a = sub + t * V;
+    if (a >= BS || i < 0) continue;
+    const int64_t o = ((i * BS + a) << m.klog) + c;
+    const T sum = split_sum<BS, T>(m, part, a, idx);
+    if (INIT) {
+      rn[t] = b[o] - sum;
+    } else {
+      rn[t] = r[o] - sum;
+      x[o] += v_in[o];
+    }
+    r[o] = rn[t];
+  }
+  if (!INIT && !has_next) return;
+  __syncthreads();  // every partial sum has been read
+#pragma unroll
+  for (int t = 0; t < (BS + 1) / 2; ++t)
+    if (sub + t * V < BS && i >= 0) part[(sub + t * V) * W + idx] = rn[t];
+  __syncthreads();
+  if (i < 0) return;
+  const double wi = w ? (double)w[i] : 1.0;
+  const T c1 = INIT ? T(0) : (T)scal[kCheb + 2 * k];
+  const T c2 = (T)((INIT ? scal[kInvTheta] : scal[kCheb + 2 * k + 1]) * wi);
+  const int64_t base = (i >> 5) * (32LL * BS * BS) + (i & 31);
+  for (int a = sub; a < BS; a += V) {
+    T z = T(0);
+#pragma unroll
+    for (int q = 0; q < BS; ++q) z = fma(__ldg(dinv + base + 32 * (a * BS + q)), part[q * W + idx], z);
+    const int64_t o = ((i * BS + a) << m.klog) + c;
+    d_out[o] = INIT ? c2 * z : fma(c1, v_in[o], c2 * z);
+  }
+}
+
+template <int BR, int BC, typename T>
+__global__ void __launch_bounds__(kSplitThreads) k_mtransfer_split(const SplitMap m, const int* __restrict__ sp,
+                                                                   const int* __restrict__ col,
+                                                                   const T* __restrict__ vals,
+                                                                   const int* __restrict__ srow, int64_t n,
+                                                                   const T* __restrict__ v, T* __restrict__ y,
+                                                                   int accumulate, const int* done) {
+  BAMG_DONE_RETURN
+  __shared__ T part[kSplitThreads * BR];
+  BAMG_SPLIT_THREAD
+  split_partials<BR, BC, T>(m, sp, col, vals, n, v, pos, c, sub, idx, part);
+  const int64_t i = pos < n ? row_at(srow, pos) : -1;
+  if (i < 0) return;
+  for (int a = sub; a < BR; a += 1 << m.vlog) {
+    const T sum = split_sum<BR, T>(m, part, a, idx);
+    const int64_t o = ((i * BR + a) << m.klog) + c;
+    y[o] = accumulate ? y[o] + sum : sum;
+  }
+}
+
 template <typename T>
 __global__ void k_maxpy(int64_t m, const T* __restrict__ d, T* __restrict__ x, const int* done) {
   BAMG_DONE_RETURN
@@ -472,6 +604,31 @@ MPtrs<T> mptrs(Level& L, MultiLevel& W) {
           f ? (const T*)(const void*)L.dinv32 : (const T*)(const void*)L.dinv, pick(L.A), pick(L.P), pick(L.R)};
 }
 
+// Whether a matrix's multi-vector kernels run in the split form, and its
+// mapping.  The unsplit form's 4-column threads fill n kp / 128 warps; below
+// two per SM sub-partition (1,216) the kernels wait on the longest row instead
+// of the FP64 pipes (1,331 rows x 16 columns, 27 6x6 blocks: 177 us unsplit,
+// 37 us split).  FP64 3x3 products also use the integer pipes (fixed.cuh)
+// and stay unsplit down to 256 warps.  A row is shared by as many threads as
+// it takes to reach four warps per sub-partition, at most one per block.  A
+// matrix set to one lane per row is never split: its columns are then summed
+// as the single-vector kernels sum them.
+template <typename T>
+bool split_map(const bamg_bsr* M, int kp, SplitMap& m) {
+  const int vec = sizeof(T) == 4 ? M->vec32 : M->vec, split = sizeof(T) == 4 ? M->split32 : M->split;
+  if ((vec <= 1 && split == 0) || M->nbr == 0) return false;
+  const bool fx = sizeof(T) == 8 && M->br == 3 && M->bc == 3;
+  if (M->nbr * kp / 128 >= (fx ? 256 : 1216)) return false;
+  const int64_t blocks = std::max<int64_t>(1, M->nnzb / M->nbr);
+  m.klog = ilog2(kp);
+  m.vlog = 1;
+  while (M->nbr * kp / 32 << m.vlog < 2432 && (2 << m.vlog) <= blocks && (kp << (m.vlog + 1)) <= kSplitThreads) ++m.vlog;
+  m.rlog = std::max(0, 8 - m.klog - m.vlog);  // CTAs of 256 threads, 512 for kp x 2^vlog = 512
+  return true;
+}
+unsigned split_grid(int64_t n, const SplitMap& m) { return (unsigned)((n + (1 << m.rlog) - 1) >> m.rlog); }
+unsigned split_block(const SplitMap& m) { return 1u << (m.klog + m.vlog + m.rlog); }
+
 template <int BS, typename T>
 Status msmooth_down(bamg_mg* mg, int l, int kp, const int* done, cudaStream_t st) {
   Level& L = mg->levels[l];
@@ -483,7 +640,16 @@ Status msmooth_down(bamg_mg* mg, int l, int kp, const int* done, cudaStream_t st
   const int m = mg->opts.cheb_degree;
   { k_mcheb_init<BS, T><<<g, 256, 0, st>>>(L.n, glog, kp, p.b, p.r, p.d0, p.x, p.dinv, L.weights, sc, done); BAMG_COUNT_LAUNCH; }
   T* d[2] = {p.d0, p.d1};
+  SplitMap sm;
+  const bool split = split_map<T>(A, kp, sm);
   for (int k = 0; k < m; ++k) {
+    if (split) {
+      k_mcheb_split<BS, T, false><<<split_grid(L.n, sm), split_block(sm), 0, st>>>(
+          sm, A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, d[k & 1], nullptr, d[(k + 1) & 1], p.x, p.r,
+          p.dinv, L.weights, sc, k, k + 1 < m ? 1 : 0, done);
+      BAMG_COUNT_LAUNCH;
+      continue;
+    }
     k_mcheb_step<BS, T><<<g, 256, 0, st>>>(A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, glog, kp, d[k & 1], d[(k + 1) & 1],
                                            p.x, p.r, p.dinv, L.weights, sc, k, k + 1 < m ? 1 : 0, done);
     BAMG_COUNT_LAUNCH;
@@ -501,10 +667,27 @@ Status msmooth_up(bamg_mg* mg, int l, int kp, const int* done, cudaStream_t st) 
   const unsigned g = grid_for(L.n << glog);
   const double* sc = mg->scal + (int64_t)l * kScalarsPerLevel;
   const int m = mg->opts.cheb_degree;
-  { k_mcheb_rinit<BS, T><<<g, 256, 0, st>>>(A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, glog, kp, p.x, p.b, p.r, p.d0,
-                                            p.dinv, L.weights, sc, done); BAMG_COUNT_LAUNCH; }
+  SplitMap sm;
+  const bool split = split_map<T>(A, kp, sm);
+  if (split) {
+    k_mcheb_split<BS, T, true><<<split_grid(L.n, sm), split_block(sm), 0, st>>>(
+        sm, A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, p.x, p.b, p.d0, nullptr, p.r, p.dinv, L.weights,
+        sc, 0, 1, done);
+    BAMG_COUNT_LAUNCH;
+  } else {
+    k_mcheb_rinit<BS, T><<<g, 256, 0, st>>>(A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, glog, kp, p.x, p.b, p.r, p.d0,
+                                            p.dinv, L.weights, sc, done);
+    BAMG_COUNT_LAUNCH;
+  }
   T* d[2] = {p.d0, p.d1};
   for (int k = 0; k + 1 < m; ++k) {
+    if (split) {
+      k_mcheb_split<BS, T, false><<<split_grid(L.n, sm), split_block(sm), 0, st>>>(
+          sm, A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, d[k & 1], nullptr, d[(k + 1) & 1], p.x, p.r,
+          p.dinv, L.weights, sc, k, 1, done);
+      BAMG_COUNT_LAUNCH;
+      continue;
+    }
     k_mcheb_step<BS, T><<<g, 256, 0, st>>>(A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, glog, kp, d[k & 1], d[(k + 1) & 1],
                                            p.x, p.r, p.dinv, L.weights, sc, k, 1, done);
     BAMG_COUNT_LAUNCH;
@@ -519,6 +702,14 @@ template <int BR, int BC, typename T>
 Status mtransfer(const bamg_bsr* M, const T* vals, const T* v, T* y, int kp, int accumulate, const int* done,
                  cudaStream_t st) {
   if (M->nbr == 0) return Status{};
+  SplitMap sm;
+  if (split_map<T>(M, kp, sm)) {
+    k_mtransfer_split<BR, BC, T><<<split_grid(M->nbr, sm), split_block(sm), 0, st>>>(
+        sm, M->slice_ptr, M->sell_col, vals, M->slot_row, M->nbr, v, y, accumulate, done);
+    BAMG_COUNT_LAUNCH;
+    BAMG_CUDA(cudaGetLastError());
+    return Status{};
+  }
   const int glog = ilog2(kp / 4);
   { k_mtransfer<BR, BC, T><<<grid_for(M->nbr << glog), 256, 0, st>>>(M->slice_ptr, M->sell_col, vals, M->slot_row,
                                                                   M->nbr, glog, kp, v, y, accumulate, done); BAMG_COUNT_LAUNCH; }

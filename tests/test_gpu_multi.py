@@ -207,3 +207,25 @@ def test_spmm_fp32_matches_oracle_products(ne, k):
             assert rel(got[:, j], y.cpu().numpy().astype(np.float64)) <= 2e-6
     finally:
         gp.close()
+
+
+@pytest.mark.parametrize("precision,tol", [(B.BAMG_FP64, TOL64), (B.BAMG_FP32, 1e-5)])
+@pytest.mark.parametrize("aggregation,ne,ks", [(B.BAMG_AGG_GEOMETRIC, 13, (3, 8, 32)), (B.BAMG_AGG_MIS, 12, (16,)),
+                                               (B.BAMG_AGG_GEOMETRIC, 21, (4, 20))])
+def test_split_rows_give_the_unsplit_cycle(precision, tol, aggregation, ne, ks):
+    """Matrices with few rows share each row's blocks among threads unless set
+    to one lane per row; both sum the same products in another order (TOL64 in
+    FP64; in FP32 a few hundred roundings of 6e-8)."""
+    gp = GpuProblem(ne, precision=precision, aggregation=aggregation)
+    try:
+        for k in ks:
+            Bh = dev(rhs(gp.mesh, k, 40))
+            X, Y = torch.zeros_like(Bh), torch.zeros_like(Bh)
+            B.bamg_mg_set_lanes(gp.ctx, gp.mg, 4)
+            B.bamg_mg_vcycle_multi(gp.ctx, gp.mg, Bh, X, k)
+            B.bamg_mg_set_lanes(gp.ctx, gp.mg, 1)
+            B.bamg_mg_vcycle_multi(gp.ctx, gp.mg, Bh, Y, k)
+            for j in range(k):
+                assert rel(X[:, j].cpu().numpy(), Y[:, j].cpu().numpy()) <= tol, (k, j)
+    finally:
+        gp.close()
