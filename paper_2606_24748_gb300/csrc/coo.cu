@@ -70,33 +70,55 @@ __global__ void k_coo_sum(const int* __restrict__ seg, const int* __restrict__ p
   if (vals32) vals32[a] = (float)sum;
 }
 
-// The same sum with one thread per storage slot (slice order) and all B
-// elements of its block: every store of a warp then writes 32 consecutive
-// slots of one element (coalesced), and each contribution is read as one run
-// of B values.  The slot's contributions are contiguous in sperm (slots in
-// slice order, each slot's in input order), so the sum order is that of
-// k_coo_sum.  Padding slots have none and are left alone.
+// The same sum with one lane per storage slot (slice order) and all B elements
+// of its block: every store of a warp then writes 32 consecutive slots of one
+// element (coalesced).  The slot's contributions are contiguous in sperm
+// (slots in slice order, each slot's in input order), so the sum order is that
+// of k_coo_sum.  Padding slots have none and are left alone.
+// A contribution is B consecutive values, so a lane that read its own would
+// have each of a warp's B loads touch 32 lines, and L1's tag rate, not HBM,
+// would set the pace (0.53 ms per 64^3 assembly).  A round's 32 contributions
+// are instead read by the whole warp, 32 consecutive values of the round at a
+// time (4 to 5 lines a load), and passed through shared memory; the lanes read
+// them back B values apart (B odd: no bank conflicts).
 template <int B>
 __global__ void __launch_bounds__(128) k_coo_sum_slots(const int* __restrict__ soff, const int* __restrict__ sperm,
                                                        const double* __restrict__ v, int64_t nslots,
                                                        double* __restrict__ vals, float* __restrict__ vals32,
                                                        int add, int* __restrict__ err) {
+  __shared__ double stage[4][32 * B];
   const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (s >= nslots) return;
-  const int c0 = soff[s], c1 = soff[s + 1];
-  if (c0 == c1 && !add) return;
+  if (s >= nslots) return;  // whole warps: slots are multiples of 32
+  const int lane = threadIdx.x & 31;
+  double* mine = stage[threadIdx.x >> 5];
+  const int c0 = soff[s], n = soff[s + 1] - c0;
+  const int rounds = __reduce_max_sync(0xffffffffu, n);
+  if (rounds == 0 && !add) return;
   double acc[B];
   const int64_t base = (s >> 5) * (32LL * B) + (s & 31);
-  if (c0 < c1) {
-    const double* p0 = v + (int64_t)__ldg(sperm + c0) * B;
+  // the first contribution starts the sum: FP64 adds run at two per clock per SM
+  int p = n > 0 ? __ldg(sperm + c0) : -1;
+  for (int c = 0; c < rounds; ++c) {
+    const int next = c + 1 < n ? __ldg(sperm + c0 + c + 1) : -1;
+    double got[B];
 #pragma unroll
-    for (int e = 0; e < B; ++e) acc[e] = __ldg(p0 + e);
-    for (int c = c0 + 1; c < c1; ++c) {
-      const double* p = v + (int64_t)__ldg(sperm + c) * B;
-#pragma unroll
-      for (int e = 0; e < B; ++e) acc[e] += __ldg(p + e);
+    for (int t = 0; t < B; ++t) {
+      const int f = t * 32 + lane, src = f / B;
+      const int ps = __shfl_sync(0xffffffffu, p, src);
+      got[t] = ps >= 0 ? __ldg(v + (int64_t)ps * B + (f - src * B)) : 0.0;
     }
-  } else {
+    __syncwarp();  // the previous round has been read
+#pragma unroll
+    for (int t = 0; t < B; ++t) mine[t * 32 + lane] = got[t];
+    __syncwarp();
+    if (c < n) {
+#pragma unroll
+      for (int e = 0; e < B; ++e) acc[e] = c == 0 ? mine[lane * B + e] : acc[e] + mine[lane * B + e];
+    }
+    p = next;
+  }
+  if (n == 0) {
+    if (!add) return;
 #pragma unroll
     for (int e = 0; e < B; ++e) acc[e] = 0.0;
   }
@@ -105,6 +127,7 @@ __global__ void __launch_bounds__(128) k_coo_sum_slots(const int* __restrict__ s
   for (int e = 0; e < B; ++e) {
     double sum = acc[e];
     if (add) sum += vals[base + 32 * e];
+    // NaN / Inf by the exponent bits (integer pipe)
     bad |= (__double_as_longlong(sum) & 0x7FF0000000000000ll) == 0x7FF0000000000000ll;
     vals[base + 32 * e] = sum;
     if (vals32) vals32[base + 32 * e] = (float)sum;
