@@ -2,6 +2,7 @@
 // from the finest level), shared by the SpMV and the cycle's transfer.
 #pragma once
 
+#include "device.cuh"
 #include "internal.h"
 
 namespace bamg {
@@ -25,6 +26,10 @@ __device__ __forceinline__ void row_blocks_split(const int* __restrict__ slice_p
   static_assert(VB >= 2, "the block split takes two or more warps");
   const int c0 = __ldg(slice_ptr + s), c1 = __ldg(slice_ptr + s + 1);
   TA acc[BR];
+  if constexpr (std::is_same<TM, double>::value && std::is_same<TX, double>::value) {
+    // on the FP64 and the integer pipes together (fixed.cuh)
+    row_sums_fx<BR, BC, VB>(c0 + w, c1, col, vals, x, lane, acc);
+  } else {
 #pragma unroll
   for (int r = 0; r < BR; ++r) acc[r] = TA(0);
   for (int c = c0 + w; c < c1; c += VB) {
@@ -42,6 +47,7 @@ __device__ __forceinline__ void row_blocks_split(const int* __restrict__ slice_p
     for (int r = 0; r < BR; ++r)
 #pragma unroll
       for (int q = 0; q < BC; ++q) acc[r] = fma((TA)blk[r * BC + q], xv[q], acc[r]);
+  }
   }
   __shared__ TA part[VB][BR][32];
 #pragma unroll

@@ -32,13 +32,13 @@ __device__ __forceinline__ double warp_sum(double v) {
 // Matrix values and columns are streamed (evict-first); x is gathered
 // through the read-only path, where neighbouring rows hit the same lines.
 // `row` is the thread's row; `sub` its lane within the row's group.
-// FP64 products of 3x3 blocks (the finest operator) are formed on the FP64
-// and the integer pipes together (fixed.cuh): the FP64 pipe alone bounds the
+// FP64 products of 3x3 and 3x6 blocks (the finest operator and prolongator)
+// are formed on the FP64 and the integer pipes together (fixed.cuh): the FP64 pipe alone bounds the
 // 64^3 operator (7.19 M blocks) at 107 us, HBM at 81.  Measured there: y = A x
 // 128 -> 104 us, the fused Chebyshev step 134 -> 112 us.
 template <int BR, int BC, typename TM, typename TX>
 constexpr bool fx_product() {
-  return BR == 3 && BC == 3 && std::is_same<TM, double>::value && std::is_same<TX, double>::value;
+  return BR == 3 && (BC == 3 || BC == 6) && std::is_same<TM, double>::value && std::is_same<TX, double>::value;
 }
 
 template <int BR, int BC, int V, typename TM, typename TA, typename TX>
@@ -65,10 +65,8 @@ template <int BR, int BC, int V>
 __device__ __forceinline__ void row_sums_fx(int c0, int c1, const int* __restrict__ col,
                                             const double* __restrict__ vals, const double* __restrict__ x, int lane,
                                             double (&acc)[BR]) {
-  using Row = FxRow<BR, BC>;
-  Row row;
-  row.init();
-  int left = Row::kCarry, carries = 0;
+  FxSum<BR, BC> sum;
+  sum.init();
 #pragma unroll 1
   for (int c = c0; c < c1; c += V) {
     const int j = __ldcs(col + (int64_t)c * 32 + lane);
@@ -78,23 +76,9 @@ __device__ __forceinline__ void row_sums_fx(int c0, int c1, const int* __restric
     for (int e = 0; e < BR * BC; ++e) blk[e] = __ldcs(v + 32 * e);
 #pragma unroll
     for (int q = 0; q < BC; ++q) xv[q] = __ldg(x + (int64_t)j * BC + q);
-    FxBlock<BR, BC> a;
-    a.cut(blk);
-    row.add(blk, a, xv);
-    if (--left == 0) {
-      left = Row::kCarry;
-      row.carry();
-      if ((++carries & 1) == 0) row.flush();
-    }
+    sum.add(blk, xv);
   }
-  row.carry();
-  row.flush();
-  if (row.valid()) {
-#pragma unroll
-    for (int r = 0; r < BR; ++r) acc[r] = row.acc[r];
-  } else {
-    row_sums<BR, BC, V, double, double, double>(c0, c1, col, vals, x, lane, acc);
-  }
+  if (!sum.finish(acc)) row_sums<BR, BC, V, double, double, double>(c0, c1, col, vals, x, lane, acc);
 }
 
 template <int BR, int BC, int V, typename TM, typename TA, typename TX>

@@ -176,4 +176,34 @@ struct FxRow {
   }
 };
 
+// One row's sums over a stream of blocks.
+template <int BR, int BC>
+struct FxSum {
+  FxRow<BR, BC> row;
+  int left, carries;
+  __device__ __forceinline__ void init() {
+    row.init();
+    left = FxRow<BR, BC>::kCarry;
+    carries = 0;
+  }
+  __device__ __forceinline__ void add(const double (&v)[BR * BC], const double (&x)[BC]) {
+    FxBlock<BR, BC> a;
+    a.cut(v);
+    row.add(v, a, x);
+    if (--left == 0) {
+      left = FxRow<BR, BC>::kCarry;
+      row.carry();
+      if ((++carries & 1) == 0) row.flush();
+    }
+  }
+  // False: the values are not covered, and the sums have to be formed by FP64 FMA.
+  __device__ __forceinline__ bool finish(double (&out)[BR]) {
+    row.carry();
+    row.flush();
+#pragma unroll
+    for (int r = 0; r < BR; ++r) out[r] = row.acc[r];
+    return row.valid();
+  }
+};
+
 }  // namespace bamg

@@ -18,6 +18,93 @@
 
 namespace bamg {
 
+// Column c of the sum over the list entries [s0, s1) of A_ik P_kJ.
+template <int BS, int BSP, typename T>
+__device__ __forceinline__ void stage1_column(int s0, int s1, const int* __restrict__ ea, const int* __restrict__ ep,
+                                              const T* __restrict__ Avals, const T* __restrict__ Pblk, int c,
+                                              T (&acc)[BS]) {
+#pragma unroll
+  for (int r = 0; r < BS; ++r) acc[r] = T(0);
+  for (int s = s0; s < s1; ++s) {
+    const int64_t aslot = __ldg(ea + s);
+    const int64_t pb = __ldg(ep + s);
+    T p[BS];
+#pragma unroll
+    for (int q = 0; q < BS; ++q) p[q] = __ldg(Pblk + pb * (BS * BSP) + q * BSP + c);
+    const T* a = Avals + (aslot >> 5) * (32LL * BS * BS) + (aslot & 31);
+#pragma unroll
+    for (int r = 0; r < BS; ++r)
+#pragma unroll
+      for (int q = 0; q < BS; ++q) acc[r] = fma(__ldg(a + 32 * (r * BS + q)), p[q], acc[r]);
+  }
+}
+
+// Column c of the sum of P_iI^T Z_iJ.
+template <int BS, int BSP, typename T>
+__device__ __forceinline__ void stage2_column(int s0, int s1, const int* __restrict__ ep, const int* __restrict__ ez,
+                                              const T* __restrict__ Pblk, const T* __restrict__ Z, int c,
+                                              T (&acc)[BSP]) {
+#pragma unroll
+  for (int u = 0; u < BSP; ++u) acc[u] = T(0);
+  for (int s = s0; s < s1; ++s) {
+    const int64_t pb = __ldg(ep + s);
+    const int64_t z = __ldg(ez + s);
+    T zc[BS];
+#pragma unroll
+    for (int r = 0; r < BS; ++r) zc[r] = __ldg(Z + z * (BS * BSP) + r * BSP + c);
+    const T* p = Pblk + pb * (BS * BSP);
+#pragma unroll
+    for (int r = 0; r < BS; ++r)
+#pragma unroll
+      for (int u = 0; u < BSP; ++u) acc[u] = fma(__ldg(p + r * BSP + u), zc[r], acc[u]);
+  }
+}
+
+// The same columns with FP64 products on both pipes (fixed.cuh); false where
+// the values are not covered and the forms above have to be taken.
+template <int BS, int BSP>
+__device__ __forceinline__ bool stage1_column_fx(int s0, int s1, const int* __restrict__ ea,
+                                                 const int* __restrict__ ep, const double* __restrict__ Avals,
+                                                 const double* __restrict__ Pblk, int c, double (&acc)[BS]) {
+  FxSum<BS, BS> sum;
+  sum.init();
+#pragma unroll 1
+  for (int s = s0; s < s1; ++s) {
+    const int64_t aslot = __ldg(ea + s);
+    const int64_t pb = __ldg(ep + s);
+    double a[BS * BS], p[BS];
+    const double* ap = Avals + (aslot >> 5) * (32LL * BS * BS) + (aslot & 31);
+#pragma unroll
+    for (int e = 0; e < BS * BS; ++e) a[e] = __ldg(ap + 32 * e);
+#pragma unroll
+    for (int q = 0; q < BS; ++q) p[q] = __ldg(Pblk + pb * (BS * BSP) + q * BSP + c);
+    sum.add(a, p);
+  }
+  return sum.finish(acc);
+}
+
+template <int BS, int BSP>
+__device__ __forceinline__ bool stage2_column_fx(int s0, int s1, const int* __restrict__ ep,
+                                                 const int* __restrict__ ez, const double* __restrict__ Pblk,
+                                                 const double* __restrict__ Z, int c, double (&acc)[BSP]) {
+  FxSum<BSP, BS> sum;
+  sum.init();
+#pragma unroll 1
+  for (int s = s0; s < s1; ++s) {
+    const int64_t pb = __ldg(ep + s);
+    const int64_t z = __ldg(ez + s);
+    double p[BSP * BS], zc[BS];
+#pragma unroll
+    for (int r = 0; r < BS; ++r)
+#pragma unroll
+      for (int u = 0; u < BSP; ++u) p[u * BS + r] = __ldg(Pblk + pb * (BS * BSP) + r * BSP + u);
+#pragma unroll
+    for (int r = 0; r < BS; ++r) zc[r] = __ldg(Z + z * (BS * BSP) + r * BSP + c);
+    sum.add(p, zc);
+  }
+  return sum.finish(acc);
+}
+
 template <int BS, int BSP, typename T>
 __global__ void __launch_bounds__(256) k_ptap_stage1(int64_t n1, const int* __restrict__ item_z,
                                                      const int* __restrict__ off, const int* __restrict__ ea,
@@ -31,20 +118,12 @@ __global__ void __launch_bounds__(256) k_ptap_stage1(int64_t n1, const int* __re
   const int64_t item = warp * G + g;
   if (item >= n1) return;
   T acc[BS];
-#pragma unroll
-  for (int r = 0; r < BS; ++r) acc[r] = T(0);
   const int s0 = __ldg(off + item), s1 = __ldg(off + item + 1);
-  for (int s = s0; s < s1; ++s) {
-    const int64_t aslot = __ldg(ea + s);
-    const int64_t pb = __ldg(ep + s);
-    T p[BS];
-#pragma unroll
-    for (int q = 0; q < BS; ++q) p[q] = __ldg(Pblk + pb * (BS * BSP) + q * BSP + c);
-    const T* a = Avals + (aslot >> 5) * (32LL * BS * BS) + (aslot & 31);
-#pragma unroll
-    for (int r = 0; r < BS; ++r)
-#pragma unroll
-      for (int q = 0; q < BS; ++q) acc[r] = fma(__ldg(a + 32 * (r * BS + q)), p[q], acc[r]);
+  if constexpr (std::is_same<T, double>::value) {
+    if (!stage1_column_fx<BS, BSP>(s0, s1, ea, ep, Avals, Pblk, c, acc))
+      stage1_column<BS, BSP, T>(s0, s1, ea, ep, Avals, Pblk, c, acc);
+  } else {
+    stage1_column<BS, BSP, T>(s0, s1, ea, ep, Avals, Pblk, c, acc);
   }
   const int64_t z = __ldg(item_z + item);
 #pragma unroll
@@ -66,20 +145,12 @@ __global__ void __launch_bounds__(256) k_ptap_stage2(int64_t n2, const int* __re
   const int64_t item = warp * G + g;
   if (item >= n2) return;
   T acc[BSP];
-#pragma unroll
-  for (int u = 0; u < BSP; ++u) acc[u] = T(0);
   const int s0 = __ldg(off + item), s1 = __ldg(off + item + 1);
-  for (int s = s0; s < s1; ++s) {
-    const int64_t pb = __ldg(ep + s);
-    const int64_t z = __ldg(ez + s);
-    T zc[BS];
-#pragma unroll
-    for (int r = 0; r < BS; ++r) zc[r] = __ldg(Z + z * (BS * BSP) + r * BSP + c);
-    const T* p = Pblk + pb * (BS * BSP);
-#pragma unroll
-    for (int r = 0; r < BS; ++r)
-#pragma unroll
-      for (int u = 0; u < BSP; ++u) acc[u] = fma(__ldg(p + r * BSP + u), zc[r], acc[u]);
+  if constexpr (std::is_same<T, double>::value) {
+    if (!stage2_column_fx<BS, BSP>(s0, s1, ep, ez, Pblk, Z, c, acc))
+      stage2_column<BS, BSP, T>(s0, s1, ep, ez, Pblk, Z, c, acc);
+  } else {
+    stage2_column<BS, BSP, T>(s0, s1, ep, ez, Pblk, Z, c, acc);
   }
   const int64_t slot = __ldg(item_slot + item);
   T* o = Ac + (slot >> 5) * (32LL * BC) + (slot & 31);

@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(256) k_spmm(const int* __restrict__ slice_ptr,
 // X and Y aligned to four elements): each block value is loaded once for four
 // vectors.
 template <int BR, int BC, typename T>
-__global__ void __launch_bounds__(256, 2) k_spmm4(const int* __restrict__ slice_ptr, const int* __restrict__ col,
+__global__ void __launch_bounds__(256, BC == 6 ? 1 : 2) k_spmm4(const int* __restrict__ slice_ptr, const int* __restrict__ col,
                                                const T* __restrict__ vals, const int* __restrict__ srow,
                                                const T* __restrict__ X, T* __restrict__ Y, int64_t nbr, int k) {
   const int G = k >> 2;

@@ -43,7 +43,7 @@ def within(got, ref, scale=1.0):
     return np.all(np.abs(got.reshape(y.shape).astype(np.longdouble) / scale - y) <= n * 2.0 ** -52 * (mag + 2.5 * top))
 
 
-@pytest.mark.parametrize("bs", [(3, 3)])
+@pytest.mark.parametrize("bs", [(3, 3), (3, 6), (6, 3)])
 def test_products_at_carry_and_flush_lengths(bs):
     rng = np.random.default_rng(5)
     lengths = [1, 19, 20, 21, 39, 40, 41, 60, 80, 81, 120, 0, 2, 7] + [27] * 40
@@ -58,7 +58,7 @@ def test_products_at_carry_and_flush_lengths(bs):
         ref = reference(bi, bj, v, x, nbr)
         xd = torch.from_numpy(x).cuda()
         single = torch.full((nbr * bs[0],), 7.0, dtype=torch.float64, device="cuda")
-        for lanes in (4, 32, 1):
+        for lanes in ((-264, -272, -288) if bs == (6, 3) else ()) + (4, 32, 1):
             B.bamg_bsr_set_lanes(ctx, A, lanes)
             B.bamg_bsr_spmv(ctx, A, xd, single)
             assert within(single.cpu().numpy(), ref), lanes
@@ -79,8 +79,7 @@ def test_products_at_carry_and_flush_lengths(bs):
         B.bamg_ctx_destroy(ctx)
 
 
-@pytest.mark.parametrize("bs", [(3, 3)])
-@pytest.mark.parametrize("lanes", [1, 4])
+@pytest.mark.parametrize("bs,lanes", [((3, 3), 1), ((3, 3), 4), ((3, 6), 1), ((6, 3), -264)])
 def test_values_outside_the_scales(bs, lanes):
     """Infinities, NaN, subnormals, the largest and smallest magnitudes and
     zero blocks beside huge x give what FP64 multiply-adds give."""
@@ -92,8 +91,8 @@ def test_values_outside_the_scales(bs, lanes):
     try:
         bi, bj, v = operator(rng, lengths, nbc, bs, 1.0)
         x = rng.standard_normal(nbc * bs[1])
-        v[9 * 3 + 2, 1, 1] = np.inf
-        v[9 * 5 + 1, 2, 0] = np.nan
+        v[9 * 3 + 2, -2, 1] = np.inf
+        v[9 * 5 + 1, -1, 0] = np.nan
         v[9 * 7:9 * 8] *= 1e-300
         v[9 * 9:9 * 10] *= 2.0 ** 900
         v[9 * 11:9 * 12] *= 2.0 ** -1060
@@ -124,4 +123,63 @@ def test_values_outside_the_scales(bs, lanes):
         assert not got[13].any()
     finally:
         B.bamg_bsr_destroy(A)
+        B.bamg_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("bs,bsp", [(3, 6), (6, 6), (3, 3)])
+@pytest.mark.parametrize("symmetric", [0, 1])
+def test_galerkin_product_at_carry_and_flush_lengths(bs, bsp, symmetric):
+    """P^T A P against extended precision, with gather lists of 1 to some 100
+    pairs: 2^-52 per product, twice, on at most 300 products of entries within
+    a factor of about 8 of their root mean square stays below 1e-12 normwise."""
+    rng = np.random.default_rng(bs + bsp)
+    n, nc = 120, 4
+    hit = rng.random((n, n)) < np.linspace(0.02, 0.9, n)[:, None]
+    hit = hit | hit.T | np.eye(n, dtype=bool)
+    hp = rng.random((n, nc)) < np.array([0.9, 0.5, 0.2, 0.03])
+    hp[:, 0] |= ~hp.any(1)
+    bi, bj = (t.astype(np.int32) for t in np.nonzero(hit))
+    pi, pj = (t.astype(np.int32) for t in np.nonzero(hp))
+    A = np.zeros((n, bs, n, bs))
+    A[bi, :, bj, :] = rng.standard_normal((bi.size, bs, bs))
+    A = (A.reshape(n * bs, n * bs) + A.reshape(n * bs, n * bs).T).reshape(n, bs, n, bs)
+    v, pv = A[bi, :, bj, :], rng.standard_normal((pi.size, bs, bsp))
+    P = np.zeros((n, bs, nc, bsp))
+    P[pi, :, pj, :] = pv
+    Pl, Al = P.reshape(n * bs, -1).astype(np.longdouble), A.reshape(n * bs, -1).astype(np.longdouble)
+    want = (Pl.T @ (Al @ Pl)).astype(np.float64)
+    ctx = B.bamg_ctx_create(torch.cuda.current_stream())
+    Ah, Ph = B.bamg_bsr_create(ctx, bs, bs, n, n), B.bamg_bsr_create(ctx, bs, bsp, n, nc)
+    plan = Ac = None
+    try:
+        for M, i, j, w in ((Ah, bi, bj, v), (Ph, pi, pj, pv)):
+            B.bamg_bsr_coo_preallocate(ctx, M, torch.from_numpy(i).cuda(), torch.from_numpy(j).cuda())
+            B.bamg_bsr_coo_set_values(ctx, M, torch.from_numpy(np.ascontiguousarray(w)).cuda(), 0)
+        B.bamg_bsr_set_symmetric(ctx, Ah, symmetric)
+        plan, Ac = B.bamg_ptap_symbolic(ctx, Ah, Ph)
+        B.bamg_ptap_numeric(ctx, plan, Ah, Ph, Ac)
+        info = B.bamg_bsr_info(Ac)
+        rp = torch.empty(info["nbr"] + 1, dtype=torch.int32, device="cuda")
+        ci = torch.empty(info["nnzb"], dtype=torch.int32, device="cuda")
+        vals = torch.empty((info["nnzb"], bsp, bsp), dtype=torch.float64, device="cuda")
+        B.bamg_bsr_get_pattern(ctx, Ac, rp, ci)
+        B.bamg_bsr_get_values(ctx, Ac, vals)
+        rows = np.repeat(np.arange(nc), np.diff(rp.cpu().numpy()))
+        got = np.zeros((nc, bsp, nc, bsp))
+        got[rows, :, ci.cpu().numpy(), :] = vals.cpu().numpy()
+        assert np.linalg.norm(got.reshape(want.shape) - want) <= 1e-12 * np.linalg.norm(want)
+        # a value outside the scales goes through FP64 multiply-adds
+        v[0, -1, -1] = np.nan
+        B.bamg_bsr_coo_set_values(ctx, Ah, torch.from_numpy(np.ascontiguousarray(v)).cuda(), 0)
+        B.bamg_ptap_numeric(ctx, plan, Ah, Ph, Ac)
+        B.bamg_bsr_get_values(ctx, Ac, vals)
+        assert torch.isnan(vals).any()
+        with pytest.raises(B.BamgError):
+            B.bamg_ctx_sync(ctx)  # the assembly reports the NaN it wrote
+    finally:
+        if plan is not None:
+            B.bamg_ptap_destroy(plan)
+            B.bamg_bsr_destroy(Ac)
+        B.bamg_bsr_destroy(Ph)
+        B.bamg_bsr_destroy(Ah)
         B.bamg_ctx_destroy(ctx)
