@@ -743,7 +743,7 @@ __global__ void k_cg_first(int64_t m, const double* __restrict__ r, const double
 
 // q = A p, alpha = rz / (p.q)
 template <int V>
-__global__ void __launch_bounds__(256, 4) k_cg_Ap(const int* __restrict__ sp, const int* __restrict__ col,
+__global__ void __launch_bounds__(256, 3) k_cg_Ap(const int* __restrict__ sp, const int* __restrict__ col,
                                                        const double* __restrict__ vals, const int* __restrict__ srow,
                                                        int64_t n, int64_t nthreads,
                                                        const double* __restrict__ p, double* __restrict__ q,
@@ -846,7 +846,7 @@ __global__ void k_cg_p(int64_t m, const double* __restrict__ z, double* __restri
 
 // ||b - A x||^2 into s->pq (final true residual)
 template <int V>
-__global__ void __launch_bounds__(256, 4) k_true_residual(const int* __restrict__ sp, const int* __restrict__ col,
+__global__ void __launch_bounds__(256, 3) k_true_residual(const int* __restrict__ sp, const int* __restrict__ col,
                                                                const double* __restrict__ vals,
                                                                const int* __restrict__ srow, int64_t n,
                                                                int64_t nthreads, const double* __restrict__ x,

@@ -35,7 +35,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // FP64 products of 3x3 and 3x6 blocks (the finest operator and prolongator)
 // are formed on the FP64 and the integer pipes together (fixed.cuh): the FP64 pipe alone bounds the
 // 64^3 operator (7.19 M blocks) at 107 us, HBM at 81.  Measured there: y = A x
-// 128 -> 104 us, the fused Chebyshev step 134 -> 112 us.
+// 128 -> 104 us, and 95 with the loads a block ahead (80 registers).
 template <int BR, int BC, typename TM, typename TX>
 constexpr bool fx_product() {
   return BR == 3 && (BC == 3 || BC == 6) && std::is_same<TM, double>::value && std::is_same<TX, double>::value;
@@ -67,16 +67,39 @@ __device__ __forceinline__ void row_sums_fx(int c0, int c1, const int* __restric
                                             double (&acc)[BR]) {
   FxSum<BR, BC> sum;
   sum.init();
-#pragma unroll 1
-  for (int c = c0; c < c1; c += V) {
-    const int j = __ldcs(col + (int64_t)c * 32 + lane);
+  double blk[BR * BC], xv[BC];
+  auto load = [&](int c, int j) {
     const double* v = vals + (int64_t)c * (32 * BR * BC) + lane;
-    double blk[BR * BC], xv[BC];
 #pragma unroll
     for (int e = 0; e < BR * BC; ++e) blk[e] = __ldcs(v + 32 * e);
 #pragma unroll
     for (int q = 0; q < BC; ++q) xv[q] = __ldg(x + (int64_t)j * BC + q);
-    sum.add(blk, xv);
+  };
+  if constexpr (BR * BC == 9) {
+    // a block ahead (3x3; two larger blocks do not fit the registers): the next block's values and x are requested before this
+    // one's products (its column one block earlier still)
+    int next = c0 < c1 ? __ldcs(col + (int64_t)c0 * 32 + lane) : 0;
+    if (c0 < c1) load(c0, next);
+    if (c0 + V < c1) next = __ldcs(col + (int64_t)(c0 + V) * 32 + lane);
+#pragma unroll 1
+    for (int c = c0; c < c1; c += V) {
+      double b[BR * BC], xb[BC];
+#pragma unroll
+      for (int e = 0; e < BR * BC; ++e) b[e] = blk[e];
+#pragma unroll
+      for (int q = 0; q < BC; ++q) xb[q] = xv[q];
+      if (c + V < c1) {
+        load(c + V, next);
+        if (c + 2 * V < c1) next = __ldcs(col + (int64_t)(c + 2 * V) * 32 + lane);
+      }
+      sum.add(b, xb);
+    }
+  } else {
+#pragma unroll 1
+    for (int c = c0; c < c1; c += V) {
+      load(c, __ldcs(col + (int64_t)c * 32 + lane));
+      sum.add(blk, xv);
+    }
   }
   if (!sum.finish(acc)) row_sums<BR, BC, V, double, double, double>(c0, c1, col, vals, x, lane, acc);
 }

@@ -279,7 +279,7 @@ __global__ void k_start_vector(double* __restrict__ v, int64_t n) {
 // One power step w_out = D^-1 A (w_in / ||w_in||) with D the block diagonal
 // (dinv) or the scalar diagonal; ||w_out|| goes to *norm_out.
 template <int BS, int V, typename TM>
-__global__ void __launch_bounds__(256, fx_product<BS, BS, TM, double>() ? 4 : 8) k_power_step(const int* __restrict__ slice_ptr,
+__global__ void __launch_bounds__(256, fx_product<BS, BS, TM, double>() ? 3 : 8) k_power_step(const int* __restrict__ slice_ptr,
                                                             const int* __restrict__ col, const TM* __restrict__ vals,
                                                             const int* __restrict__ srow,
                                                             const int* __restrict__ diag_slot,
