@@ -94,6 +94,55 @@ struct FxBlock {
   }
 };
 
+// A block as it is kept where many threads read it: the FP64 rows, the others'
+// limbs and the largest high word, in 16-byte words.
+template <int BR, int BC>
+struct FxCut {
+  using Block = FxBlock<BR, BC>;
+  static constexpr int F = Block::R0 * BC, N = Block::N;
+  static constexpr int kWords = (2 * F + 2 * N + 1 + 3) / 4;  // 16-byte words
+  __device__ __forceinline__ static void pack(const double (&v)[BR * BC], uint4 (&out)[kWords]) {
+    unsigned w[4 * kWords];
+#pragma unroll
+    for (int e = 0; e < F; ++e) {
+      w[2 * e] = fx_bits(v[e]).lo;
+      w[2 * e + 1] = fx_bits(v[e]).hi;
+    }
+    Block a;
+    a.cut(v);
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+      w[2 * (F + e)] = (unsigned)a.h[e];
+      w[2 * (F + e) + 1] = (unsigned)a.l[e];
+    }
+    w[2 * (F + N)] = a.top;
+#pragma unroll
+    for (int k = 2 * (F + N) + 1; k < 4 * kWords; ++k) w[k] = 0;
+#pragma unroll
+    for (int k = 0; k < kWords; ++k) out[k] = make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
+  }
+  __device__ __forceinline__ static void load(const uint4* __restrict__ p, double (&v)[F], Block& a) {
+    unsigned w[4 * kWords];
+#pragma unroll
+    for (int k = 0; k < kWords; ++k) {
+      const uint4 q = __ldg(p + k);
+      w[4 * k] = q.x;
+      w[4 * k + 1] = q.y;
+      w[4 * k + 2] = q.z;
+      w[4 * k + 3] = q.w;
+    }
+#pragma unroll
+    for (int e = 0; e < F; ++e) v[e] = __hiloint2double((int)w[2 * e + 1], (int)w[2 * e]);
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+      a.h[e] = (int)w[2 * (F + e)];
+      a.l[e] = (int)w[2 * (F + e) + 1];
+    }
+    a.top = w[2 * (F + N)];
+    a.exp = max((int)(a.top >> 20), kFxMinExp);
+  }
+};
+
 // Sums of one row (all its components) over its blocks for one vector.
 template <int BR, int BC>
 struct FxRow {
@@ -114,7 +163,10 @@ struct FxRow {
     E = 0;
     amax = xmax = 0;
   }
-  __device__ __forceinline__ void add(const double (&v)[BR * BC], const FxBlock<BR, BC>& a, const double (&x)[BC]) {
+  // v: the block's values, at least its first R0 rows
+  template <int M>
+  __device__ __forceinline__ void add(const double (&v)[M], const FxBlock<BR, BC>& a, const double (&x)[BC]) {
+    static_assert(M >= R0 * BC, "the FP64 rows come first");
 #pragma unroll
     for (int r = 0; r < R0; ++r)
 #pragma unroll
@@ -189,6 +241,10 @@ struct FxSum {
   __device__ __forceinline__ void add(const double (&v)[BR * BC], const double (&x)[BC]) {
     FxBlock<BR, BC> a;
     a.cut(v);
+    add(v, a, x);
+  }
+  template <int M>
+  __device__ __forceinline__ void add(const double (&v)[M], const FxBlock<BR, BC>& a, const double (&x)[BC]) {
     row.add(v, a, x);
     if (--left == 0) {
       left = FxRow<BR, BC>::kCarry;

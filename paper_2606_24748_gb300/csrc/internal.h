@@ -143,8 +143,8 @@ struct bamg_bsr {
 // Z = A P block by block, stage 2 forms A_c = P^T Z; both gather, for each
 // output block, a fixed list of input block pairs (built once by the symbolic
 // phase), so the numeric phase has no atomics and a fixed summation order.
-// Output blocks are processed in order of decreasing list length so the
-// lane groups of a warp carry equal work.
+// Output blocks are processed by decreasing list length (stage 1: within runs
+// of rows) so the lane groups of a warp carry equal work.
 struct bamg_ptap {
   bamg_ctx* ctx = nullptr;
   const bamg_bsr* A = nullptr;
@@ -162,11 +162,16 @@ struct bamg_ptap {
   // stage 2: items (A_c blocks, upper triangle if symmetric), lists of (P block, Z block)
   int64_t n2 = 0, e2 = 0;
   int *s2_slot = nullptr, *s2_tslot = nullptr, *s2_off = nullptr, *s2_p = nullptr, *s2_z = nullptr;
+  int rounds1 = 1;  // stage 1: rounds of items per CTA
   // work buffers and the state-gated prolongator-side cache (P in block order)
   double* Z = nullptr;
   float* Z32 = nullptr;
   double* Pblk = nullptr;
   float* Pblk32 = nullptr;
+  // blocks cut for the FP64 stages (fixed.cuh): A's by slot, cut for every
+  // product, and P's transposed, with the state-gated cache
+  unsigned *Acut = nullptr, *Pcut = nullptr;
+  float* Apad = nullptr;  // A's FP32 blocks by slot, padded to 16 bytes, for every FP32 product
   uint64_t pblk_version = ~0ull, pblk32_version = ~0ull;
   uint64_t pblk_refreshes = 0;
   int prof_stage1 = -1, prof_stage2 = -1;  // profiling slots of the two stages (-1: none)

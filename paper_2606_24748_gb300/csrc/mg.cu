@@ -872,6 +872,13 @@ static Status mg_setup_impl(bamg_mg* mg, bamg_bsr* A, const double* coords, cons
   return Status{};
 }
 
+// The mixed form's products run in FP64 during setup only.
+static void trim_plans(bamg_mg* mg) {
+  if (mg->opts.precision != BAMG_FP32) return;
+  for (auto& L : mg->levels)
+    if (L.plan) dfree(L.plan->Acut, mg->ctx->stream);
+}
+
 // The coarsest factorisation needs only the last Galerkin product and is a
 // chain of small dependent steps that leaves most of the GPU idle, while the
 // smoother refresh (block inverses, power iterations) keeps the FP64 pipes
@@ -1008,6 +1015,7 @@ bamg_status bamg_mg_setup(bamg_ctx* ctx, bamg_bsr* A, const double* coords, cons
   mg->opts = o;
   Status s = mg_setup_impl(mg, A, coords, dirichlet);
   if (s.ok()) s = mg_update_impl(mg);
+  trim_plans(mg);
   if (s.ok() && o.autotune) {
     for (auto& L : mg->levels) {
       if (s.ok()) s = bsr_autotune(L.A, nullptr);
@@ -1034,6 +1042,7 @@ bamg_status bamg_mg_resetup(bamg_mg* mg) {
       BAMG_TRY(smooth_level(mg, l));
       BAMG_TRY(ptap_run(mg->levels[l].plan, mg->levels[l].A, mg->levels[l].P, mg->levels[l + 1].A, BAMG_FP64, true));
     }
+    trim_plans(mg);
     BAMG_TRY(mg_update_impl(mg));
     return check_device_error(mg->ctx);
   };

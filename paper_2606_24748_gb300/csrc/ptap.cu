@@ -18,7 +18,70 @@
 
 namespace bamg {
 
-// Column c of the sum over the list entries [s0, s1) of A_ik P_kJ.
+// Values of a block in the FP32 stages' block-ordered copies: padded to whole
+// 16-byte words, so that a block's values come in a quarter of the loads (the
+// stages are bound by L1's rate of scattered loads: 51^3, stage 1 462 -> 420 us
+// with the copy, stage 2 215 -> 183).  The FP64 copies of P stay unpadded.
+template <typename T>
+__host__ __device__ constexpr int block_pitch(int n) { return sizeof(T) == 4 ? (n + 3) / 4 * 4 : n; }
+
+template <int N>
+__device__ __forceinline__ void load_block(const float* __restrict__ p, float (&v)[N]) {
+#pragma unroll
+  for (int k = 0; k < (N + 3) / 4; ++k) {
+    const float4 q = __ldg(reinterpret_cast<const float4*>(p) + k);
+    const float w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (4 * k + e < N) v[4 * k + e] = w[e];
+  }
+}
+
+// Column c of the sum over the list entries [s0, s1) of A_ik P_kJ (FP32).
+template <int BS, int BSP>
+__device__ __forceinline__ void stage1_column32(int s0, int s1, const int* __restrict__ ea,
+                                                const int* __restrict__ ep, const float* __restrict__ Ablk,
+                                                const float* __restrict__ Pblk, int c, float (&acc)[BS]) {
+#pragma unroll
+  for (int r = 0; r < BS; ++r) acc[r] = 0.0f;
+#pragma unroll 2
+  for (int s = s0; s < s1; ++s) {
+    const int64_t aslot = __ldg(ea + s);
+    const int64_t pb = __ldg(ep + s);
+    float a[BS * BS], p[BS];
+    load_block<BS * BS>(Ablk + aslot * block_pitch<float>(BS * BS), a);
+#pragma unroll
+    for (int q = 0; q < BS; ++q) p[q] = __ldg(Pblk + pb * block_pitch<float>(BS * BSP) + q * BSP + c);
+#pragma unroll
+    for (int r = 0; r < BS; ++r)
+#pragma unroll
+      for (int q = 0; q < BS; ++q) acc[r] = fma(a[r * BS + q], p[q], acc[r]);
+  }
+}
+
+// Column c of the sum of P_iI^T Z_iJ (FP32).
+template <int BS, int BSP>
+__device__ __forceinline__ void stage2_column32(int s0, int s1, const int* __restrict__ ep,
+                                                const int* __restrict__ ez, const float* __restrict__ Pblk,
+                                                const float* __restrict__ Z, int c, float (&acc)[BSP]) {
+#pragma unroll
+  for (int u = 0; u < BSP; ++u) acc[u] = 0.0f;
+#pragma unroll 2
+  for (int s = s0; s < s1; ++s) {
+    const int64_t pb = __ldg(ep + s);
+    const int64_t z = __ldg(ez + s);
+    float p[BS * BSP], zc[BS];
+    load_block<BS * BSP>(Pblk + pb * block_pitch<float>(BS * BSP), p);
+#pragma unroll
+    for (int r = 0; r < BS; ++r) zc[r] = __ldg(Z + z * (BS * BSP) + r * BSP + c);
+#pragma unroll
+    for (int r = 0; r < BS; ++r)
+#pragma unroll
+      for (int u = 0; u < BSP; ++u) acc[u] = fma(p[r * BSP + u], zc[r], acc[u]);
+  }
+}
+
+// The same columns by FP64 FMA, from the sliced storage.
 template <int BS, int BSP, typename T>
 __device__ __forceinline__ void stage1_column(int s0, int s1, const int* __restrict__ ea, const int* __restrict__ ep,
                                               const T* __restrict__ Avals, const T* __restrict__ Pblk, int c,
@@ -39,7 +102,6 @@ __device__ __forceinline__ void stage1_column(int s0, int s1, const int* __restr
   }
 }
 
-// Column c of the sum of P_iI^T Z_iJ.
 template <int BS, int BSP, typename T>
 __device__ __forceinline__ void stage2_column(int s0, int s1, const int* __restrict__ ep, const int* __restrict__ ez,
                                               const T* __restrict__ Pblk, const T* __restrict__ Z, int c,
@@ -61,73 +123,153 @@ __device__ __forceinline__ void stage2_column(int s0, int s1, const int* __restr
 }
 
 // The same columns with FP64 products on both pipes (fixed.cuh); false where
-// the values are not covered and the forms above have to be taken.
+// the values are not covered and the forms above have to be taken.  The six
+// lanes of an output block share A_ik (stage 1) and P_iI (stage 2), so these
+// are read cut, from block-ordered copies: a lane that cut A_ik itself read it
+// as nine sectors of the sliced storage and repeated the others' work.
 template <int BS, int BSP>
 __device__ __forceinline__ bool stage1_column_fx(int s0, int s1, const int* __restrict__ ea,
-                                                 const int* __restrict__ ep, const double* __restrict__ Avals,
+                                                 const int* __restrict__ ep, const uint4* __restrict__ Acut,
                                                  const double* __restrict__ Pblk, int c, double (&acc)[BS]) {
+  using Cut = FxCut<BS, BS>;
   FxSum<BS, BS> sum;
   sum.init();
 #pragma unroll 1
   for (int s = s0; s < s1; ++s) {
     const int64_t aslot = __ldg(ea + s);
     const int64_t pb = __ldg(ep + s);
-    double a[BS * BS], p[BS];
-    const double* ap = Avals + (aslot >> 5) * (32LL * BS * BS) + (aslot & 31);
-#pragma unroll
-    for (int e = 0; e < BS * BS; ++e) a[e] = __ldg(ap + 32 * e);
+    double f[Cut::F], p[BS];
+    typename Cut::Block a;
+    Cut::load(Acut + aslot * Cut::kWords, f, a);
 #pragma unroll
     for (int q = 0; q < BS; ++q) p[q] = __ldg(Pblk + pb * (BS * BSP) + q * BSP + c);
-    sum.add(a, p);
+    sum.add(f, a, p);
   }
   return sum.finish(acc);
 }
 
 template <int BS, int BSP>
 __device__ __forceinline__ bool stage2_column_fx(int s0, int s1, const int* __restrict__ ep,
-                                                 const int* __restrict__ ez, const double* __restrict__ Pblk,
+                                                 const int* __restrict__ ez, const uint4* __restrict__ Pcut,
                                                  const double* __restrict__ Z, int c, double (&acc)[BSP]) {
+  using Cut = FxCut<BSP, BS>;
   FxSum<BSP, BS> sum;
   sum.init();
 #pragma unroll 1
   for (int s = s0; s < s1; ++s) {
     const int64_t pb = __ldg(ep + s);
     const int64_t z = __ldg(ez + s);
-    double p[BSP * BS], zc[BS];
-#pragma unroll
-    for (int r = 0; r < BS; ++r)
-#pragma unroll
-      for (int u = 0; u < BSP; ++u) p[u * BS + r] = __ldg(Pblk + pb * (BS * BSP) + r * BSP + u);
+    double f[Cut::F], zc[BS];
+    typename Cut::Block p;
+    Cut::load(Pcut + pb * Cut::kWords, f, p);
 #pragma unroll
     for (int r = 0; r < BS; ++r) zc[r] = __ldg(Z + z * (BS * BSP) + r * BSP + c);
-    sum.add(p, zc);
+    sum.add(f, p, zc);
   }
   return sum.finish(acc);
 }
 
+// Cut copies: A's blocks by storage slot, and P's blocks transposed, in block
+// order.  A lane packs a block; the warp writes its 32 blocks as one run.
+template <int BR, int BC, int W>
+__device__ __forceinline__ void write_cut(const uint4 (&w)[W], int64_t first, int64_t n, uint4* stage,
+                                          uint4* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 0; k < W; ++k) stage[lane * W + k] = w[k];
+  __syncwarp();
+  for (int k = lane; k < (int)min((int64_t)32, n - first) * W; k += 32) out[first * W + k] = stage[k];
+}
+
+template <int BS>
+__global__ void __launch_bounds__(64) k_cut_slots(int64_t nslots, const double* __restrict__ vals,
+                                                  uint4* __restrict__ out) {
+  using Cut = FxCut<BS, BS>;
+  __shared__ uint4 stage[2][32 * Cut::kWords];
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= nslots) return;  // whole warps
+  double v[BS * BS];
+#pragma unroll
+  for (int e = 0; e < BS * BS; ++e) v[e] = __ldcs(vals + vidx<BS * BS>(t, e));
+  uint4 w[Cut::kWords];
+  Cut::pack(v, w);
+  write_cut<BS, BS, Cut::kWords>(w, t & ~31LL, nslots, stage[threadIdx.x >> 5], out);
+}
+
+// FP32 blocks by storage slot, padded (block_pitch).
+template <int BS>
+__global__ void __launch_bounds__(128) k_pad_slots(int64_t nslots, const float* __restrict__ vals,
+                                                   float4* __restrict__ out) {
+  constexpr int N = BS * BS, W = block_pitch<float>(N) / 4;
+  __shared__ float4 stage[4][32 * W];
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= nslots) return;  // whole warps
+  float v[4 * W];
+#pragma unroll
+  for (int e = 0; e < 4 * W; ++e) v[e] = e < N ? __ldcs(vals + vidx<N>(t, e)) : 0.0f;
+  const int lane = threadIdx.x & 31;
+  float4* mine = stage[threadIdx.x >> 5];
+#pragma unroll
+  for (int k = 0; k < W; ++k) mine[lane * W + k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < W; ++k) out[(t - lane) * W + k * 32 + lane] = mine[k * 32 + lane];
+}
+
+// FP32 blocks in block order, padded, from the FP64 ones.
+__global__ void k_pad_blocks(int64_t nblk, int n, int pitch, const double* __restrict__ src, float* __restrict__ dst) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= nblk * pitch) return;
+  const int64_t b = t / pitch;
+  const int e = (int)(t - b * pitch);
+  dst[t] = e < n ? (float)src[b * n + e] : 0.0f;
+}
+
+template <int BS, int BSP>
+__global__ void __launch_bounds__(64) k_cut_transposed(int64_t nblk, const double* __restrict__ Pblk,
+                                                       uint4* __restrict__ out) {
+  using Cut = FxCut<BSP, BS>;
+  __shared__ uint4 stage[2][32 * Cut::kWords];
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t first = t & ~31LL;
+  if (first >= nblk) return;  // whole warps
+  const int64_t b = min(t, nblk - 1);
+  double v[BSP * BS];
+#pragma unroll
+  for (int r = 0; r < BS; ++r)
+#pragma unroll
+    for (int u = 0; u < BSP; ++u) v[u * BS + r] = __ldg(Pblk + b * (BS * BSP) + r * BSP + u);
+  uint4 w[Cut::kWords];
+  Cut::pack(v, w);
+  write_cut<BSP, BS, Cut::kWords>(w, first, nblk, stage[threadIdx.x >> 5], out);
+}
+
 template <int BS, int BSP, typename T>
-__global__ void __launch_bounds__(256) k_ptap_stage1(int64_t n1, const int* __restrict__ item_z,
+__global__ void __launch_bounds__(256) k_ptap_stage1(int64_t n1, int rounds, const int* __restrict__ item_z,
                                                      const int* __restrict__ off, const int* __restrict__ ea,
                                                      const int* __restrict__ ep, const T* __restrict__ Avals,
-                                                     const T* __restrict__ Pblk, T* __restrict__ Z) {
+                                                     const T* __restrict__ Pblk, const uint4* __restrict__ Acut,
+                                                     T* __restrict__ Z) {
   constexpr int G = 32 / BSP;
-  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const int g = lane / BSP, c = lane - g * BSP;
   if (g >= G) return;
-  const int64_t item = warp * G + g;
-  if (item >= n1) return;
-  T acc[BS];
-  const int s0 = __ldg(off + item), s1 = __ldg(off + item + 1);
-  if constexpr (std::is_same<T, double>::value) {
-    if (!stage1_column_fx<BS, BSP>(s0, s1, ea, ep, Avals, Pblk, c, acc))
-      stage1_column<BS, BSP, T>(s0, s1, ea, ep, Avals, Pblk, c, acc);
-  } else {
-    stage1_column<BS, BSP, T>(s0, s1, ea, ep, Avals, Pblk, c, acc);
-  }
-  const int64_t z = __ldg(item_z + item);
+  const int64_t first = (int64_t)blockIdx.x * rounds * 8 * G;
+  for (int t = 0; t < rounds; ++t) {
+    const int64_t item = first + (t * 8 + (threadIdx.x >> 5)) * G + g;
+    if (item >= n1) return;
+    T acc[BS];
+    const int s0 = __ldg(off + item), s1 = __ldg(off + item + 1);
+    if constexpr (std::is_same<T, double>::value) {
+      if (!stage1_column_fx<BS, BSP>(s0, s1, ea, ep, Acut, Pblk, c, acc))
+        stage1_column<BS, BSP, T>(s0, s1, ea, ep, Avals, Pblk, c, acc);
+    } else {
+      stage1_column32<BS, BSP>(s0, s1, ea, ep, Avals, Pblk, c, acc);
+    }
+    const int64_t z = __ldg(item_z + item);
 #pragma unroll
-  for (int r = 0; r < BS; ++r) Z[z * (BS * BSP) + r * BSP + c] = acc[r];
+    for (int r = 0; r < BS; ++r) Z[z * (BS * BSP) + r * BSP + c] = acc[r];
+  }
 }
 
 template <int BS, int BSP, typename T>
@@ -135,22 +277,22 @@ __global__ void __launch_bounds__(256) k_ptap_stage2(int64_t n2, const int* __re
                                                      const int* __restrict__ item_tslot,
                                                      const int* __restrict__ off, const int* __restrict__ ep,
                                                      const int* __restrict__ ez, const T* __restrict__ Pblk,
-                                                     const T* __restrict__ Z, T* __restrict__ Ac) {
+                                                     const uint4* __restrict__ Pcut, const T* __restrict__ Z,
+                                                     T* __restrict__ Ac) {
   constexpr int G = 32 / BSP;
   constexpr int BC = BSP * BSP;
-  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const int g = lane / BSP, c = lane - g * BSP;
   if (g >= G) return;
-  const int64_t item = warp * G + g;
+  const int64_t item = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * G + g;
   if (item >= n2) return;
   T acc[BSP];
   const int s0 = __ldg(off + item), s1 = __ldg(off + item + 1);
   if constexpr (std::is_same<T, double>::value) {
-    if (!stage2_column_fx<BS, BSP>(s0, s1, ep, ez, Pblk, Z, c, acc))
+    if (!stage2_column_fx<BS, BSP>(s0, s1, ep, ez, Pcut, Z, c, acc))
       stage2_column<BS, BSP, T>(s0, s1, ep, ez, Pblk, Z, c, acc);
   } else {
-    stage2_column<BS, BSP, T>(s0, s1, ep, ez, Pblk, Z, c, acc);
+    stage2_column32<BS, BSP>(s0, s1, ep, ez, Pblk, Z, c, acc);
   }
   const int64_t slot = __ldg(item_slot + item);
   T* o = Ac + (slot >> 5) * (32LL * BC) + (slot & 31);
@@ -158,22 +300,32 @@ __global__ void __launch_bounds__(256) k_ptap_stage2(int64_t n2, const int* __re
   for (int u = 0; u < BSP; ++u) o[32 * (u * BSP + c)] = acc[u];
   const int64_t ts = __ldg(item_tslot + item);
   if (ts >= 0) {
-    T* t = Ac + (ts >> 5) * (32LL * BC) + (ts & 31);
+    T* tv = Ac + (ts >> 5) * (32LL * BC) + (ts & 31);
 #pragma unroll
-    for (int u = 0; u < BSP; ++u) t[32 * (c * BSP + u)] = acc[u];
+    for (int u = 0; u < BSP; ++u) tv[32 * (c * BSP + u)] = acc[u];
   }
 }
 
-// Stable order of items by decreasing list length (counting sort).
-static std::vector<int> order_by_work(const std::vector<int>& off) {
+// Stage 1: items of one CTA, rounds x (8 warps x 32 / bs_p items).  A CTA takes a
+// run of items in row order, sorted by list length, so that the items that
+// share operand blocks (one row's and its neighbours') meet in one L1 while the
+// lane groups of a warp still carry equal work; sorted over all items, every
+// block comes from L2 or HBM once per list it is in (64^3: 2.27 -> 1.93 ms).
+// More rounds share more but leave fewer CTAs: eight where each of 152 SMs
+// still gets eight CTAs.  Stage 2's lists differ too much in length within a
+// run (0.63 ms sorted over all items, 1.07 in runs).
+static int item_rounds(int64_t items, int bsp) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(8, items / (8 * (32 / bsp) * 152 * 8)));
+}
+
+// Stable order of items by decreasing list length within runs of `window`.
+static std::vector<int> order_by_work(const std::vector<int>& off, int64_t window) {
   const int64_t n = (int64_t)off.size() - 1;
-  int maxlen = 0;
-  for (int64_t i = 0; i < n; ++i) maxlen = std::max(maxlen, off[i + 1] - off[i]);
-  std::vector<int64_t> start(maxlen + 2, 0);
-  for (int64_t i = 0; i < n; ++i) start[maxlen - (off[i + 1] - off[i]) + 1]++;
-  for (int l = 0; l <= maxlen; ++l) start[l + 1] += start[l];
   std::vector<int> order((size_t)n);
-  for (int64_t i = 0; i < n; ++i) order[start[maxlen - (off[i + 1] - off[i])]++] = (int)i;
+  std::iota(order.begin(), order.end(), 0);
+  for (int64_t w = 0; w < n; w += window)
+    std::stable_sort(order.begin() + w, order.begin() + std::min(n, w + window),
+                     [&](int a, int b) { return off[a + 1] - off[a] > off[b + 1] - off[b]; });
   return order;
 }
 
@@ -210,6 +362,9 @@ void ptap_release(bamg_ptap* p) {
   dfree(p->Z32, st);
   dfree(p->Pblk, st);
   dfree(p->Pblk32, st);
+  dfree(p->Acut, st);
+  dfree(p->Pcut, st);
+  dfree(p->Apad, st);
 }
 
 Status ptap_build(bamg_bsr* A, bamg_bsr* P, bool want_ac, bamg_ptap** plan_out, bamg_bsr** Ac_out) {
@@ -293,7 +448,8 @@ Status ptap_build(bamg_bsr* A, bamg_bsr* P, bool want_ac, bamg_ptap** plan_out, 
     pl->n1 = pl->nz;
     pl->e1 = (int64_t)la.size();
     {
-      std::vector<int> order = order_by_work(off1), noff, na, np;
+      pl->rounds1 = item_rounds(pl->n1, bsp);
+      std::vector<int> order = order_by_work(off1, pl->rounds1 * 8 * (32 / bsp)), noff, na, np;
       permute_lists(order, off1, la, lp, noff, na, np);
       BAMG_TRY(upload(&pl->s1_z, order, st));
       BAMG_TRY(upload(&pl->s1_off, noff, st));
@@ -392,7 +548,7 @@ Status ptap_build(bamg_bsr* A, bamg_bsr* P, bool want_ac, bamg_ptap** plan_out, 
     }
     pl->n2 = (int64_t)item_ac.size();
     pl->e2 = (int64_t)l2p.size();
-    std::vector<int> order = order_by_work(off2), noff, np, nz;
+    std::vector<int> order = order_by_work(off2, std::max<int64_t>(1, pl->n2)), noff, np, nz;
     permute_lists(order, off2, l2p, l2z, noff, np, nz);
     std::vector<int> os(order.size()), ots(order.size());
     for (size_t t = 0; t < order.size(); ++t) {
@@ -423,32 +579,37 @@ Status ptap_build(bamg_bsr* A, bamg_bsr* P, bool want_ac, bamg_ptap** plan_out, 
 template <typename T>
 static Status run_stages(bamg_ptap* pl, const T* Avals, const T* Pblk, T* Z, T* Acvals, bool stage2) {
   cudaStream_t st = pl->ctx->stream;
+  const uint4* Acut = (const uint4*)pl->Acut;
+  const uint4* Pcut = (const uint4*)pl->Pcut;
   const int G = 32 / pl->bsp;
-  auto blocks_for = [&](int64_t items) { return (unsigned)((items + (int64_t)G * 8 - 1) / ((int64_t)G * 8)); };
+  auto blocks_for = [&](int64_t items, int rounds) {
+    const int64_t per = (int64_t)rounds * 8 * G;
+    return (unsigned)((items + per - 1) / per);
+  };
   if (pl->n1 > 0) {
-    const unsigned b = blocks_for(pl->n1);
+    const unsigned b = blocks_for(pl->n1, pl->rounds1);
     const int pm = prof_begin(pl->ctx, pl->prof_stage1, st);
     if (pl->bs == 3 && pl->bsp == 6)
-      { k_ptap_stage1<3, 6, T><<<b, 256, 0, st>>>(pl->n1, pl->s1_z, pl->s1_off, pl->s1_a, pl->s1_p, Avals, Pblk, Z); BAMG_COUNT_LAUNCH; }
+      { k_ptap_stage1<3, 6, T><<<b, 256, 0, st>>>(pl->n1, pl->rounds1, pl->s1_z, pl->s1_off, pl->s1_a, pl->s1_p, Avals, Pblk, Acut, Z); BAMG_COUNT_LAUNCH; }
     else if (pl->bs == 6 && pl->bsp == 6)
-      { k_ptap_stage1<6, 6, T><<<b, 256, 0, st>>>(pl->n1, pl->s1_z, pl->s1_off, pl->s1_a, pl->s1_p, Avals, Pblk, Z); BAMG_COUNT_LAUNCH; }
+      { k_ptap_stage1<6, 6, T><<<b, 256, 0, st>>>(pl->n1, pl->rounds1, pl->s1_z, pl->s1_off, pl->s1_a, pl->s1_p, Avals, Pblk, Acut, Z); BAMG_COUNT_LAUNCH; }
     else
-      { k_ptap_stage1<3, 3, T><<<b, 256, 0, st>>>(pl->n1, pl->s1_z, pl->s1_off, pl->s1_a, pl->s1_p, Avals, Pblk, Z); BAMG_COUNT_LAUNCH; }
+      { k_ptap_stage1<3, 3, T><<<b, 256, 0, st>>>(pl->n1, pl->rounds1, pl->s1_z, pl->s1_off, pl->s1_a, pl->s1_p, Avals, Pblk, Acut, Z); BAMG_COUNT_LAUNCH; }
     prof_end(pl->ctx, pm, st);
     BAMG_CUDA(cudaGetLastError());
   }
   if (stage2 && pl->n2 > 0) {
-    const unsigned b = blocks_for(pl->n2);
+    const unsigned b = blocks_for(pl->n2, 1);
     const int pm = prof_begin(pl->ctx, pl->prof_stage2, st);
     if (pl->bs == 3 && pl->bsp == 6)
       { k_ptap_stage2<3, 6, T><<<b, 256, 0, st>>>(pl->n2, pl->s2_slot, pl->s2_tslot, pl->s2_off, pl->s2_p, pl->s2_z,
-                                                Pblk, Z, Acvals); BAMG_COUNT_LAUNCH; }
+                                                Pblk, Pcut, Z, Acvals); BAMG_COUNT_LAUNCH; }
     else if (pl->bs == 6 && pl->bsp == 6)
       { k_ptap_stage2<6, 6, T><<<b, 256, 0, st>>>(pl->n2, pl->s2_slot, pl->s2_tslot, pl->s2_off, pl->s2_p, pl->s2_z,
-                                                Pblk, Z, Acvals); BAMG_COUNT_LAUNCH; }
+                                                Pblk, Pcut, Z, Acvals); BAMG_COUNT_LAUNCH; }
     else
       { k_ptap_stage2<3, 3, T><<<b, 256, 0, st>>>(pl->n2, pl->s2_slot, pl->s2_tslot, pl->s2_off, pl->s2_p, pl->s2_z,
-                                                Pblk, Z, Acvals); BAMG_COUNT_LAUNCH; }
+                                                Pblk, Pcut, Z, Acvals); BAMG_COUNT_LAUNCH; }
     prof_end(pl->ctx, pm, st);
     BAMG_CUDA(cudaGetLastError());
   }
@@ -464,14 +625,70 @@ static Status refresh_pblk(bamg_ptap* pl, bamg_bsr* P, bool fp32) {
     if (P->vals64_stale) return make_status(BAMG_ERR_STATE, "P holds only FP32 values");
     if (!pl->Pblk) BAMG_TRY(dalloc(&pl->Pblk, ne, st));
     BAMG_TRY(launch_gather_blocks(P, P->vals, pl->Pblk, st));
+    if (pl->Ac && P->nnzb > 0) {  // the second stage's cut copy
+      const int words = pl->bs == 6 ? FxCut<6, 6>::kWords : pl->bsp == 6 ? FxCut<6, 3>::kWords : FxCut<3, 3>::kWords;
+      if (!pl->Pcut) BAMG_TRY(dalloc(&pl->Pcut, P->nnzb * words * 4, st));
+      const unsigned b = (unsigned)((P->nnzb + 63) / 64);
+      uint4* out = (uint4*)pl->Pcut;
+      if (pl->bs == 6)
+        k_cut_transposed<6, 6><<<b, 64, 0, st>>>(P->nnzb, pl->Pblk, out);
+      else if (pl->bsp == 6)
+        k_cut_transposed<3, 6><<<b, 64, 0, st>>>(P->nnzb, pl->Pblk, out);
+      else
+        k_cut_transposed<3, 3><<<b, 64, 0, st>>>(P->nnzb, pl->Pblk, out);
+      BAMG_COUNT_LAUNCH;
+      BAMG_CUDA(cudaGetLastError());
+    }
     pl->pblk_version = P->version;
     pl->pblk_refreshes++;
   }
   if (fp32 && pl->pblk32_version != P->version) {
-    if (!pl->Pblk32) BAMG_TRY(dalloc(&pl->Pblk32, ne, st));
-    BAMG_TRY(launch_to_fp32(pl->Pblk, pl->Pblk32, ne, st));
+    const int n = (int)P->block_elems(), pitch = block_pitch<float>(n);
+    if (!pl->Pblk32) BAMG_TRY(dalloc(&pl->Pblk32, P->nnzb * pitch, st));
+    if (P->nnzb > 0) {
+      k_pad_blocks<<<(unsigned)((P->nnzb * pitch + 255) / 256), 256, 0, st>>>(P->nnzb, n, pitch, pl->Pblk, pl->Pblk32);
+      BAMG_COUNT_LAUNCH;
+      BAMG_CUDA(cudaGetLastError());
+    }
     pl->pblk32_version = P->version;
   }
+  return Status{};
+}
+
+// Cut copy of A's blocks for this product (their values are new every time).
+static Status cut_operator(bamg_ptap* pl, const bamg_bsr* A) {
+  cudaStream_t st = pl->ctx->stream;
+  const int64_t n = A->nslots();
+  if (n == 0) return Status{};
+  const int words = pl->bs == 6 ? FxCut<6, 6>::kWords : FxCut<3, 3>::kWords;
+  if (!pl->Acut) BAMG_TRY(dalloc(&pl->Acut, n * words * 4, st));
+  const unsigned b = (unsigned)((n + 63) / 64);
+  const int pm = prof_begin(pl->ctx, pl->prof_stage1, st, 0);
+  if (pl->bs == 6)
+    k_cut_slots<6><<<b, 64, 0, st>>>(n, A->vals, (uint4*)pl->Acut);
+  else
+    k_cut_slots<3><<<b, 64, 0, st>>>(n, A->vals, (uint4*)pl->Acut);
+  BAMG_COUNT_LAUNCH;
+  prof_end(pl->ctx, pm, st);
+  BAMG_CUDA(cudaGetLastError());
+  return Status{};
+}
+
+// FP32 copy of A's blocks for this product, padded.
+static Status pad_operator(bamg_ptap* pl, const bamg_bsr* A) {
+  cudaStream_t st = pl->ctx->stream;
+  const int64_t n = A->nslots();
+  if (n == 0) return Status{};
+  if (!pl->Apad) BAMG_TRY(dalloc(&pl->Apad, n * block_pitch<float>(pl->bs * pl->bs), st));
+  const unsigned b = (unsigned)((n + 127) / 128);
+  const int pm = prof_begin(pl->ctx, pl->prof_stage1, st, 0);
+  if (pl->bs == 6)
+    k_pad_slots<6><<<b, 128, 0, st>>>(n, A->vals32, (float4*)pl->Apad);
+  else
+    k_pad_slots<3><<<b, 128, 0, st>>>(n, A->vals32, (float4*)pl->Apad);
+  BAMG_COUNT_LAUNCH;
+  prof_end(pl->ctx, pm, st);
+  BAMG_CUDA(cudaGetLastError());
   return Status{};
 }
 
@@ -484,10 +701,13 @@ Status ptap_run(bamg_ptap* pl, bamg_bsr* A, bamg_bsr* P, bamg_bsr* Ac, bamg_prec
   if (prec == BAMG_FP64) {
     if (A->vals64_stale) return make_status(BAMG_ERR_STATE, "A holds only FP32 values; use BAMG_FP32");
     BAMG_TRY(refresh_pblk(pl, P, false));
+    BAMG_TRY(cut_operator(pl, A));
     BAMG_TRY(run_stages<double>(pl, A->vals, pl->Pblk, pl->Z, stage2 ? Ac->vals : nullptr, stage2));
     if (stage2) {
       Ac->version++;
       Ac->vals64_stale = false;
+    } else {
+      dfree(pl->Acut, st);  // prolongator smoothing: setup only
     }
   } else if (prec == BAMG_FP32) {
     BAMG_TRY(bsr_ensure_fp32(A));
@@ -496,7 +716,8 @@ Status ptap_run(bamg_ptap* pl, bamg_bsr* A, bamg_bsr* P, bamg_bsr* Ac, bamg_prec
     if (stage2 && !Ac->vals32) BAMG_TRY(dalloc(&Ac->vals32, Ac->nslots() * Ac->block_elems(), st));
     if (stage2 && Ac->vals32 && Ac->vals32_version == ~0ull)
       BAMG_CUDA(cudaMemsetAsync(Ac->vals32, 0, sizeof(float) * Ac->nslots() * Ac->block_elems(), st));
-    BAMG_TRY(run_stages<float>(pl, A->vals32, pl->Pblk32, pl->Z32, stage2 ? Ac->vals32 : nullptr, stage2));
+    BAMG_TRY(pad_operator(pl, A));
+    BAMG_TRY(run_stages<float>(pl, pl->Apad, pl->Pblk32, pl->Z32, stage2 ? Ac->vals32 : nullptr, stage2));
     if (stage2) {
       Ac->version++;
       Ac->vals32_version = Ac->version;
