@@ -394,11 +394,10 @@ __device__ __forceinline__ void row_sums4_fx(int a0, int a1, const int* __restri
   unsigned redo = 0;  // vectors that the scales do not cover: formed by FP64 FMA, one at a time
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
-    row[e].carry();
-    row[e].flush();
-    if (!row[e].valid()) redo |= 1u << e;
+    double out[BR];
+    if (!row[e].finish(out, carries >= 2)) redo |= 1u << e;
 #pragma unroll
-    for (int r = 0; r < BR; ++r) acc[r][e] = row[e].acc[r];
+    for (int r = 0; r < BR; ++r) acc[r][e] = out[r];
   }
 #pragma unroll 1
   for (int e = 0; redo >> e; ++e) {

@@ -213,18 +213,61 @@ struct FxRow {
       mid[r] -= up << 28;
     }
   }
+  // The sums as doubles, rounded to nearest, by integer operations: an FP64
+  // conversion or add holds the SM sub-partition for 64 cycles, and a row of
+  // four blocks would spend as many of them here as on its products.  Exact in
+  // the sign; needs valid().
+  __device__ __forceinline__ double value(int r) const {
+    const unsigned long long low = ((unsigned long long)hh[r] << 28) + (unsigned long long)mid[r];
+    long long high = (hh[r] >> 36) + (mid[r] >> 63) + (low < (unsigned long long)mid[r] ? 1 : 0);
+    unsigned long long lo = low;
+    const bool neg = high < 0;
+    if (neg) {
+      lo = 0 - lo;
+      high = ~high + (lo == 0);
+    }
+    unsigned long long m = (unsigned long long)high;
+    int e = 64;
+    if (m == 0) {
+      m = lo;
+      lo = 0;
+      e = 0;
+    }
+    if (m == 0) return 0.0;
+    const int z = __clzll((long long)m);
+    m = z ? (m << z) | (lo >> (64 - z)) : m;
+    // the sum is m 2^(e - z) 2^(E - 2128)
+    const unsigned long long mant = (m >> 11) + ((m >> 10) & 1);
+    const unsigned long long bits = ((unsigned long long)(E - 2128 + 63 + e - z + 1022) << 52) + mant;
+    return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0)));
+  }
   __device__ __forceinline__ void flush() {  // after carry()
-    const double scale = __longlong_as_double((long long)(max(E, 1106) - 1105) << 52);
+    if (!covers()) amax = 0x7fffffffu;  // these sums are lost: the row is not valid
 #pragma unroll
     for (int r = 0; r < NI; ++r) {
-      acc[R0 + r] = fma(fma((double)hh[r], 268435456.0, (double)(int)mid[r]), scale, acc[R0 + r]);
+      if (covers()) acc[R0 + r] += value(r);
       hh[r] = mid[r] = 0;
     }
   }
-  // Whether acc[] is the row's product; otherwise it has to be formed by FP64 FMA.
+  // The row's sums; flushed: whether flush() has been called before.
+  __device__ __forceinline__ bool finish(double (&out)[BR], bool flushed) {  // false: not valid
+    carry();
+    const bool ok = valid();
+#pragma unroll
+    for (int r = 0; r < R0; ++r) out[r] = acc[r];
+#pragma unroll
+    for (int r = 0; r < NI; ++r) {
+      const double v = ok ? value(r) : 0.0;
+      out[R0 + r] = flushed ? acc[R0 + r] + v : v;
+    }
+    return ok;
+  }
+  // The exponent gives normal doubles (E = 0: no product yet).
+  __device__ __forceinline__ bool covers() const { return E == 0 || (unsigned)(E - 1106) < 1950u; }
+  // Whether the sums are the row's products; otherwise these have to be formed by FP64 FMA.
   __device__ __forceinline__ bool valid() const {
     auto covered = [](unsigned m) { return m == 0 || m - 0x10000000u < 0x60000000u; };
-    return covered(amax) && covered(xmax) && (E == 0 || (unsigned)(E - 1106) < 2046u);
+    return covered(amax) && covered(xmax) && covers();
   }
 };
 
@@ -254,11 +297,7 @@ struct FxSum {
   }
   // False: the values are not covered, and the sums have to be formed by FP64 FMA.
   __device__ __forceinline__ bool finish(double (&out)[BR]) {
-    row.carry();
-    row.flush();
-#pragma unroll
-    for (int r = 0; r < BR; ++r) out[r] = row.acc[r];
-    return row.valid();
+    return row.finish(out, carries >= 2);
   }
 };
 

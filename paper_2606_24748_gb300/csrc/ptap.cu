@@ -272,7 +272,9 @@ __global__ void __launch_bounds__(256) k_ptap_stage1(int64_t n1, int rounds, con
   }
 }
 
-template <int BS, int BSP, typename T>
+// S warps share an item's list, each taking a run of it; their sums meet in
+// shared memory and are added in list order (S = 1: no sharing).
+template <int BS, int BSP, int S, typename T>
 __global__ void __launch_bounds__(256) k_ptap_stage2(int64_t n2, const int* __restrict__ item_slot,
                                                      const int* __restrict__ item_tslot,
                                                      const int* __restrict__ off, const int* __restrict__ ep,
@@ -281,28 +283,48 @@ __global__ void __launch_bounds__(256) k_ptap_stage2(int64_t n2, const int* __re
                                                      T* __restrict__ Ac) {
   constexpr int G = 32 / BSP;
   constexpr int BC = BSP * BSP;
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = warp % S;
   const int g = lane / BSP, c = lane - g * BSP;
-  if (g >= G) return;
-  const int64_t item = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * G + g;
-  if (item >= n2) return;
+  const int64_t item = ((int64_t)blockIdx.x * (8 / S) + warp / S) * G + g;
+  const bool on = g < G && item < n2;
   T acc[BSP];
-  const int s0 = __ldg(off + item), s1 = __ldg(off + item + 1);
-  if constexpr (std::is_same<T, double>::value) {
-    if (!stage2_column_fx<BS, BSP>(s0, s1, ep, ez, Pcut, Z, c, acc))
-      stage2_column<BS, BSP, T>(s0, s1, ep, ez, Pblk, Z, c, acc);
-  } else {
-    stage2_column32<BS, BSP>(s0, s1, ep, ez, Pblk, Z, c, acc);
+  if (on) {
+    const int l0 = __ldg(off + item), l1 = __ldg(off + item + 1);
+    const int part = (l1 - l0 + S - 1) / S;
+    const int s0 = min(l1, l0 + sub * part), s1 = min(l1, s0 + part);
+    if constexpr (std::is_same<T, double>::value) {
+      if (!stage2_column_fx<BS, BSP>(s0, s1, ep, ez, Pcut, Z, c, acc))
+        stage2_column<BS, BSP, T>(s0, s1, ep, ez, Pblk, Z, c, acc);
+    } else {
+      stage2_column32<BS, BSP>(s0, s1, ep, ez, Pblk, Z, c, acc);
+    }
   }
+  if constexpr (S > 1) {
+    __shared__ T sums[8][BSP][32];
+#pragma unroll
+    for (int u = 0; u < BSP; ++u) sums[warp][u][lane] = on ? acc[u] : T(0);
+    __syncthreads();
+    if (!on) return;
+    // each warp finishes components sub, sub + S, ...
+#pragma unroll
+    for (int u = 0; u < BSP; ++u) {
+      if (u % S != sub) continue;
+      T t = sums[warp - sub][u][lane];
+#pragma unroll
+      for (int k = 1; k < S; ++k) t += sums[warp - sub + k][u][lane];
+      acc[u] = t;
+    }
+  }
+  if (!on) return;
   const int64_t slot = __ldg(item_slot + item);
   T* o = Ac + (slot >> 5) * (32LL * BC) + (slot & 31);
-#pragma unroll
-  for (int u = 0; u < BSP; ++u) o[32 * (u * BSP + c)] = acc[u];
   const int64_t ts = __ldg(item_tslot + item);
-  if (ts >= 0) {
-    T* tv = Ac + (ts >> 5) * (32LL * BC) + (ts & 31);
+  T* tv = Ac + (ts >> 5) * (32LL * BC) + (ts & 31);
 #pragma unroll
-    for (int u = 0; u < BSP; ++u) tv[32 * (c * BSP + u)] = acc[u];
+  for (int u = 0; u < BSP; ++u) {
+    if (u % S != sub) continue;
+    o[32 * (u * BSP + c)] = acc[u];
+    if (ts >= 0) tv[32 * (c * BSP + u)] = acc[u];
   }
 }
 
@@ -599,17 +621,34 @@ static Status run_stages(bamg_ptap* pl, const T* Avals, const T* Pblk, T* Z, T* 
     BAMG_CUDA(cudaGetLastError());
   }
   if (stage2 && pl->n2 > 0) {
-    const unsigned b = blocks_for(pl->n2, 1);
+    // The coarser the level, the fewer and the longer the lists: warps share
+    // them until there are 16 per SM sub-partition (64^3, level 1: 3,601 items
+    // are 91 CTAs and took 321 us; 12^3, level 0: 125 -> 23 us shared by eight).
+    int S = 1;
+    while (S < 8 && pl->n2 / G * S < 152 * 4 * 16) S *= 2;
+    const int64_t per = (int64_t)(8 / S) * G;
+    const unsigned b = (unsigned)((pl->n2 + per - 1) / per);
     const int pm = prof_begin(pl->ctx, pl->prof_stage2, st);
-    if (pl->bs == 3 && pl->bsp == 6)
-      { k_ptap_stage2<3, 6, T><<<b, 256, 0, st>>>(pl->n2, pl->s2_slot, pl->s2_tslot, pl->s2_off, pl->s2_p, pl->s2_z,
-                                                Pblk, Pcut, Z, Acvals); BAMG_COUNT_LAUNCH; }
-    else if (pl->bs == 6 && pl->bsp == 6)
-      { k_ptap_stage2<6, 6, T><<<b, 256, 0, st>>>(pl->n2, pl->s2_slot, pl->s2_tslot, pl->s2_off, pl->s2_p, pl->s2_z,
-                                                Pblk, Pcut, Z, Acvals); BAMG_COUNT_LAUNCH; }
-    else
-      { k_ptap_stage2<3, 3, T><<<b, 256, 0, st>>>(pl->n2, pl->s2_slot, pl->s2_tslot, pl->s2_off, pl->s2_p, pl->s2_z,
-                                                Pblk, Pcut, Z, Acvals); BAMG_COUNT_LAUNCH; }
+#define BAMG_STAGE2(A, B, N)                                                                                       \
+  k_ptap_stage2<A, B, N, T><<<b, 256, 0, st>>>(pl->n2, pl->s2_slot, pl->s2_tslot, pl->s2_off, pl->s2_p, pl->s2_z, \
+                                               Pblk, Pcut, Z, Acvals)
+#define BAMG_STAGE2_S(A, B)           \
+  switch (S) {                        \
+    case 8: BAMG_STAGE2(A, B, 8); break; \
+    case 4: BAMG_STAGE2(A, B, 4); break; \
+    case 2: BAMG_STAGE2(A, B, 2); break; \
+    default: BAMG_STAGE2(A, B, 1); break; \
+  }
+    if (pl->bs == 3 && pl->bsp == 6) {
+      BAMG_STAGE2_S(3, 6)
+    } else if (pl->bs == 6 && pl->bsp == 6) {
+      BAMG_STAGE2_S(6, 6)
+    } else {
+      BAMG_STAGE2_S(3, 3)
+    }
+#undef BAMG_STAGE2_S
+#undef BAMG_STAGE2
+    BAMG_COUNT_LAUNCH;
     prof_end(pl->ctx, pm, st);
     BAMG_CUDA(cudaGetLastError());
   }
