@@ -327,6 +327,15 @@ __device__ __forceinline__ void st4(float* p, const float (&v)[4]) {
   reinterpret_cast<float4*>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
 }
 
+// CTA size of the FP32 3x3 multi-vector kernels.  Small CTAs keep more of them
+// at different places in their rows (48^3, 16 vectors: 91 us in CTAs of 256
+// threads, 65 us in 64 with the loads a block ahead).
+constexpr int kMulti32Threads = 64;
+template <int BR, int BC, typename T>
+__host__ __device__ constexpr int multi_threads() {
+  return BR == 3 && BC == 3 && sizeof(T) == 4 ? kMulti32Threads : 256;
+}
+
 template <int BR, int BC, typename T>
 __device__ __forceinline__ void row_sums4(int a0, int a1, const int* __restrict__ col, const T* __restrict__ vals,
                                           const T* __restrict__ X, int kp, int lane, int c0, T (&acc)[BR][4]) {
@@ -334,6 +343,41 @@ __device__ __forceinline__ void row_sums4(int a0, int a1, const int* __restrict_
   for (int r = 0; r < BR; ++r)
 #pragma unroll
     for (int e = 0; e < 4; ++e) acc[r][e] = T(0);
+  if constexpr (BR == 3 && BC == 3 && sizeof(T) == 4) {
+    // a block ahead: the products are bound by the latency of column -> X
+    T blk[9], xv[3][4];
+    auto load = [&](int c, int j) {
+      const T* v = vals + (int64_t)c * (32 * 9) + lane;
+#pragma unroll
+      for (int e = 0; e < 9; ++e) blk[e] = __ldg(v + 32 * e);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) ld4(X + ((int64_t)j * 3 + q) * kp + c0, xv[q]);
+    };
+    int next = a0 < a1 ? __ldg(col + (int64_t)a0 * 32 + lane) : 0;
+    if (a0 < a1) load(a0, next);
+    if (a0 + 1 < a1) next = __ldg(col + (int64_t)(a0 + 1) * 32 + lane);
+#pragma unroll 1
+    for (int c = a0; c < a1; ++c) {
+      T b[9], x[3][4];
+#pragma unroll
+      for (int e = 0; e < 9; ++e) b[e] = blk[e];
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[q][e] = xv[q][e];
+      if (c + 1 < a1) {
+        load(c + 1, next);
+        if (c + 2 < a1) next = __ldg(col + (int64_t)(c + 2) * 32 + lane);
+      }
+#pragma unroll
+      for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[r][e] = fma(b[r * 3 + q], x[q][e], acc[r][e]);
+    }
+    return;
+  }
   for (int c = a0; c < a1; ++c) {
     const int j = __ldg(col + (int64_t)c * 32 + lane);
     const T* v = vals + (int64_t)c * (32 * BR * BC) + lane;

@@ -36,6 +36,18 @@ inline unsigned deal_grid(K kernel, int sm_count, int64_t threads) {
   const int64_t cap = std::min<int64_t>((int64_t)sm_count * per_sm, kRedGridMax);
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>((threads + 31) / 32, cap));
 }
+// The FP64 3x3 power steps (fixed.cuh): CTAs of 128 threads, six to an SM, in one
+// wave.  Small matrices spread four warp tasks to a CTA over all SMs, and the
+// coarsest factorisation, which runs beside them on another stream, finds room
+// sooner than beside CTAs of 256 threads (refresh 12^3 0.30 -> 0.24 ms; MIS
+// hierarchy step at 24^3 6.5 -> 6.0 ms).  More, shorter CTAs cost more in their
+// exits and partial sums than they balance, and the CG product, which runs
+// alone, is faster in CTAs of 256 threads (64^3: 110 against 117 us).
+constexpr int kFxRedThreads = 128;
+inline unsigned fx_red_grid(int sm_count, int64_t threads) {
+  const int64_t ctas = (threads + kFxRedThreads - 1) / kFxRedThreads;
+  return (unsigned)std::max<int64_t>(1, std::min<int64_t>(ctas, std::min<int64_t>(6LL * sm_count, kRedGridMax)));
+}
 constexpr int kRedThreads = 256;
 
 struct Status {

@@ -279,7 +279,8 @@ __global__ void k_start_vector(double* __restrict__ v, int64_t n) {
 // One power step w_out = D^-1 A (w_in / ||w_in||) with D the block diagonal
 // (dinv) or the scalar diagonal; ||w_out|| goes to *norm_out.
 template <int BS, int V, typename TM>
-__global__ void __launch_bounds__(256, fx_product<BS, BS, TM, double>() ? 3 : 8) k_power_step(const int* __restrict__ slice_ptr,
+__global__ void __launch_bounds__(fx_product<BS, BS, TM, double>() ? kFxRedThreads : 256,
+                                  fx_product<BS, BS, TM, double>() ? 6 : 8) k_power_step(const int* __restrict__ slice_ptr,
                                                             const int* __restrict__ col, const TM* __restrict__ vals,
                                                             const int* __restrict__ srow,
                                                             const int* __restrict__ diag_slot,
@@ -371,7 +372,7 @@ __global__ void __launch_bounds__(768) k_power_step_split(const int* __restrict_
 // Rayleigh quotient w^T A w / w^T D w; in block mode also the Chebyshev data
 // for the interval [lower, upper] * lambda (Saad, Alg. 12.1 coefficients).
 template <int BS, int V, typename TM>
-__global__ void __launch_bounds__(256) k_rayleigh(const int* __restrict__ slice_ptr,
+__global__ void __launch_bounds__(fx_product<BS, BS, TM, double>() ? kFxRedThreads : 256) k_rayleigh(const int* __restrict__ slice_ptr,
                                                           const int* __restrict__ col, const TM* __restrict__ vals,
                                                           const int* __restrict__ srow,
                                                           const int* __restrict__ diag_slot, int scalar_diag,
@@ -441,6 +442,7 @@ static Status power_impl(bamg_mg* mg, const bamg_bsr* A, const TM* vals, const d
   double* w[2] = {mg->power_w[0], mg->power_w[1]};
   double* norms = mg->scal + (int64_t)mg->levels.size() * kScalarsPerLevel;  // 2 scratch slots
   { k_start_vector<<<(unsigned)((n * BS + 255) / 256), 256, 0, st>>>(w[0], n * BS); BAMG_COUNT_LAUNCH; }
+  constexpr bool fx = fx_product<BS, BS, TM, double>();
   const int split = (BS == 6 && !scalar_diag) ? split_for<TM>(A) : 0;
   for (int it = 0; it < mg->opts.power_its; ++it) {
     const double* nin = it == 0 ? nullptr : norms + ((it + 1) & 1);
@@ -453,11 +455,11 @@ static Status power_impl(bamg_mg* mg, const bamg_bsr* A, const TM* vals, const d
         BAMG_COUNT_LAUNCH; })
       continue;
     }
-    BAMG_DISPATCH_V(lanes_for<TM>(A), { k_power_step<BS, V, TM><<<deal_grid(k_power_step<BS, V, TM>, ctx->sm_count, rows), 256, 0, st>>>(A->slice_ptr, A->sell_col, vals, A->slot_row, A->diag_slot, dinv,
+    BAMG_DISPATCH_V(lanes_for<TM>(A), { k_power_step<BS, V, TM><<<fx ? fx_red_grid(ctx->sm_count, rows) : deal_grid(k_power_step<BS, V, TM>, ctx->sm_count, rows), fx ? kFxRedThreads : 256, 0, st>>>(A->slice_ptr, A->sell_col, vals, A->slot_row, A->diag_slot, dinv,
                                                     scalar_diag ? 1 : 0, scalar_diag ? nullptr : wts, w[it & 1], w[(it + 1) & 1], nin,
                                                     norms + (it & 1), n, rows, ctx->d_partials, ctx->d_counters); BAMG_COUNT_LAUNCH; })
   }
-  BAMG_DISPATCH_V(lanes_for<TM>(A), { k_rayleigh<BS, V, TM><<<deal_grid(k_rayleigh<BS, V, TM>, ctx->sm_count, rows), 256, 0, st>>>(A->slice_ptr, A->sell_col, vals, A->slot_row, A->diag_slot, scalar_diag ? 1 : 0,
+  BAMG_DISPATCH_V(lanes_for<TM>(A), { k_rayleigh<BS, V, TM><<<fx ? fx_red_grid(ctx->sm_count, rows) : deal_grid(k_rayleigh<BS, V, TM>, ctx->sm_count, rows), fx ? kFxRedThreads : 256, 0, st>>>(A->slice_ptr, A->sell_col, vals, A->slot_row, A->diag_slot, scalar_diag ? 1 : 0,
                                                 scalar_diag ? nullptr : wts, w[mg->opts.power_its & 1], n, rows, ctx->d_partials,
                                                 ctx->d_counters + 1, out_scal, mg->opts.cheb_lower,
                                                 mg->opts.cheb_upper, mg->opts.cheb_degree); BAMG_COUNT_LAUNCH; })

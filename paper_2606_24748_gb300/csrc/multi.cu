@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(256) k_mcheb_init(int64_t n, int glog, int kp,
 
 // x += d_in; r -= A d_in; if has_next: d_out = c1 d_in + c2 w Dinv r
 template <int BS, typename T>
-__global__ void __launch_bounds__(256, 2) k_mcheb_step(const int* __restrict__ sp, const int* __restrict__ col,
+__global__ void __launch_bounds__(multi_threads<BS, BS, T>(), sizeof(T) == 4 ? 1 : 2) k_mcheb_step(const int* __restrict__ sp, const int* __restrict__ col,
                                                     const T* __restrict__ vals, const int* __restrict__ srow,
                                                     int64_t n, int glog, int kp,
                                                     const T* __restrict__ d_in, T* __restrict__ d_out,
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(256, 2) k_mcheb_step(const int* __restrict__ s
 
 // r = b - A x; d = w Dinv r / theta
 template <int BS, typename T>
-__global__ void __launch_bounds__(256, 2) k_mcheb_rinit(const int* __restrict__ sp, const int* __restrict__ col,
+__global__ void __launch_bounds__(multi_threads<BS, BS, T>(), sizeof(T) == 4 ? 1 : 2) k_mcheb_rinit(const int* __restrict__ sp, const int* __restrict__ col,
                                                      const T* __restrict__ vals, const int* __restrict__ srow,
                                                      int64_t n, int glog, int kp,
                                                      const T* __restrict__ x, const T* __restrict__ b,
@@ -638,6 +638,7 @@ Status msmooth_down(bamg_mg* mg, int l, int kp, const int* done, cudaStream_t st
   const unsigned g = grid_for(L.n << glog);
   const double* sc = mg->scal + (int64_t)l * kScalarsPerLevel;
   const int m = mg->opts.cheb_degree;
+  constexpr int mt = multi_threads<BS, BS, T>();
   { k_mcheb_init<BS, T><<<g, 256, 0, st>>>(L.n, glog, kp, p.b, p.r, p.d0, p.x, p.dinv, L.weights, sc, done); BAMG_COUNT_LAUNCH; }
   T* d[2] = {p.d0, p.d1};
   SplitMap sm;
@@ -650,7 +651,7 @@ Status msmooth_down(bamg_mg* mg, int l, int kp, const int* done, cudaStream_t st
       BAMG_COUNT_LAUNCH;
       continue;
     }
-    k_mcheb_step<BS, T><<<g, 256, 0, st>>>(A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, glog, kp, d[k & 1], d[(k + 1) & 1],
+    k_mcheb_step<BS, T><<<grid_for(L.n << glog, mt), mt, 0, st>>>(A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, glog, kp, d[k & 1], d[(k + 1) & 1],
                                            p.x, p.r, p.dinv, L.weights, sc, k, k + 1 < m ? 1 : 0, done);
     BAMG_COUNT_LAUNCH;
   }
@@ -664,9 +665,9 @@ Status msmooth_up(bamg_mg* mg, int l, int kp, const int* done, cudaStream_t st) 
   auto p = mptrs<T>(L, mg->multi->lv[l]);
   const bamg_bsr* A = L.A;
   const int glog = ilog2(kp / 4);
-  const unsigned g = grid_for(L.n << glog);
   const double* sc = mg->scal + (int64_t)l * kScalarsPerLevel;
   const int m = mg->opts.cheb_degree;
+  constexpr int mt = multi_threads<BS, BS, T>();
   SplitMap sm;
   const bool split = split_map<T>(A, kp, sm);
   if (split) {
@@ -675,7 +676,7 @@ Status msmooth_up(bamg_mg* mg, int l, int kp, const int* done, cudaStream_t st) 
         sc, 0, 1, done);
     BAMG_COUNT_LAUNCH;
   } else {
-    k_mcheb_rinit<BS, T><<<g, 256, 0, st>>>(A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, glog, kp, p.x, p.b, p.r, p.d0,
+    k_mcheb_rinit<BS, T><<<grid_for(L.n << glog, mt), mt, 0, st>>>(A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, glog, kp, p.x, p.b, p.r, p.d0,
                                             p.dinv, L.weights, sc, done);
     BAMG_COUNT_LAUNCH;
   }
@@ -688,7 +689,7 @@ Status msmooth_up(bamg_mg* mg, int l, int kp, const int* done, cudaStream_t st) 
       BAMG_COUNT_LAUNCH;
       continue;
     }
-    k_mcheb_step<BS, T><<<g, 256, 0, st>>>(A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, glog, kp, d[k & 1], d[(k + 1) & 1],
+    k_mcheb_step<BS, T><<<grid_for(L.n << glog, mt), mt, 0, st>>>(A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, glog, kp, d[k & 1], d[(k + 1) & 1],
                                            p.x, p.r, p.dinv, L.weights, sc, k, 1, done);
     BAMG_COUNT_LAUNCH;
   }

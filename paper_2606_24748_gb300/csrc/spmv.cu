@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(256) k_spmm(const int* __restrict__ slice_ptr,
 // X and Y aligned to four elements): each block value is loaded once for four
 // vectors.
 template <int BR, int BC, typename T>
-__global__ void __launch_bounds__(256, BC == 6 ? 1 : 2) k_spmm4(const int* __restrict__ slice_ptr, const int* __restrict__ col,
+__global__ void __launch_bounds__(multi_threads<BR, BC, T>(), sizeof(T) == 4 ? 1 : BC == 6 ? 1 : 2) k_spmm4(const int* __restrict__ slice_ptr, const int* __restrict__ col,
                                                const T* __restrict__ vals, const int* __restrict__ srow,
                                                const T* __restrict__ X, T* __restrict__ Y, int64_t nbr, int k) {
   const int G = k >> 2;
@@ -322,11 +322,12 @@ Status launch_spmm(const bamg_bsr* A, const T* vals, const T* X, T* Y, int k, cu
   const int64_t nt = A->nbr * (int64_t)k;
   if (nt == 0) return Status{};
   const bool four = k % 4 == 0 && ((uintptr_t)X % (4 * sizeof(T))) == 0 && ((uintptr_t)Y % (4 * sizeof(T))) == 0;
-  const unsigned blocks = (unsigned)(((four ? nt / 4 : nt) + 255) / 256);
+  const unsigned blocks = (unsigned)((nt + 255) / 256);
 #define BAMG_SPMM_CASE(R, C)                                                                   \
   if (A->br == R && A->bc == C) {                                                              \
+    constexpr int t4 = multi_threads<R, C, T>();                                               \
     if (four)                                                                                  \
-      { k_spmm4<R, C, T><<<blocks, 256, 0, st>>>(A->slice_ptr, A->sell_col, vals, A->slot_row, X, Y, A->nbr, k); BAMG_COUNT_LAUNCH; } \
+      { k_spmm4<R, C, T><<<(unsigned)((nt / 4 + t4 - 1) / t4), t4, 0, st>>>(A->slice_ptr, A->sell_col, vals, A->slot_row, X, Y, A->nbr, k); BAMG_COUNT_LAUNCH; } \
     else                                                                                       \
       { k_spmm<R, C, T><<<blocks, 256, 0, st>>>(A->slice_ptr, A->sell_col, vals, A->slot_row, X, Y, A->nbr, k); BAMG_COUNT_LAUNCH; } \
     BAMG_CUDA(cudaGetLastError());                                                             \
