@@ -80,9 +80,10 @@ __global__ void k_coo_sum(const int* __restrict__ seg, const int* __restrict__ p
 // would set the pace (0.53 ms per 64^3 assembly).  A round's 32 contributions
 // are instead read by the whole warp, 32 consecutive values of the round at a
 // time (4 to 5 lines a load), and passed through shared memory; the lanes read
-// them back B values apart (B odd: no bank conflicts).
+// them back B values apart (B odd: no bank conflicts).  Held to 64 registers for
+// 32 warps per SM (64^3: 398 us unbounded at 72, 370 so).
 template <int B>
-__global__ void __launch_bounds__(128) k_coo_sum_slots(const int* __restrict__ soff, const int* __restrict__ sperm,
+__global__ void __launch_bounds__(128, 8) k_coo_sum_slots(const int* __restrict__ soff, const int* __restrict__ sperm,
                                                        const double* __restrict__ v, int64_t nslots,
                                                        double* __restrict__ vals, float* __restrict__ vals32,
                                                        int add, int* __restrict__ err) {
