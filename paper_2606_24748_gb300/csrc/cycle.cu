@@ -160,14 +160,15 @@ __global__ void __launch_bounds__(768) k_cheb_step_split(const int* __restrict__
                                                          T* __restrict__ x, T* __restrict__ r,
                                                          const T* __restrict__ dinv, const float* __restrict__ w,
                                                          const double* __restrict__ scal, int k, int has_next,
-                                                         const int* done) {
+                                                         int ncta, const int* done) {
   pdl_enter();
   BAMG_DONE_RETURN
   __shared__ T rs[BS][32];
-  const int64_t s = blockIdx.x;
+  const int64_t s = blockIdx.x / ncta;
   const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31, a = wp % BS, sub = wp / BS;
   const int64_t i = row_at(srow, s * 32 + lane);
-  const T acc = row_component<BS, BS, VS, T, T, T>(sp, col, vals, d_in, s, lane, a, sub);
+  T acc;
+  if (!row_component<BS, BS, VS, T, T, T>(sp, col, vals, d_in, s, lane, a, sub, ncta, acc)) return;
   const bool lead = sub == 0 && i >= 0 && i < n;
   T ri = T(0), di = T(0);
   if (lead) {
@@ -200,14 +201,16 @@ __global__ void __launch_bounds__(768) k_cheb_rinit_split(const int* __restrict_
                                                           const T* __restrict__ x, const T* __restrict__ b,
                                                           T* __restrict__ r, T* __restrict__ d,
                                                           const T* __restrict__ dinv, const float* __restrict__ w,
-                                                          const double* __restrict__ scal, const int* done) {
+                                                          const double* __restrict__ scal, int ncta,
+                                                          const int* done) {
   pdl_enter();
   BAMG_DONE_RETURN
   __shared__ T rs[BS][32];
-  const int64_t s = blockIdx.x;
+  const int64_t s = blockIdx.x / ncta;
   const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31, a = wp % BS, sub = wp / BS;
   const int64_t i = row_at(srow, s * 32 + lane);
-  const T acc = row_component<BS, BS, VS, T, T, T>(sp, col, vals, x, s, lane, a, sub);
+  T acc;
+  if (!row_component<BS, BS, VS, T, T, T>(sp, col, vals, x, s, lane, a, sub, ncta, acc)) return;
   const bool lead = sub == 0 && i >= 0 && i < n;
   T ri = T(0);
   if (lead) {
@@ -229,13 +232,14 @@ template <int BR, int BC, int VS, typename T>
 __global__ void __launch_bounds__(768) k_transfer_split(const int* __restrict__ sp, const int* __restrict__ col,
                                                         const T* __restrict__ vals, const int* __restrict__ srow,
                                                         int64_t n, const T* __restrict__ v, T* __restrict__ y,
-                                                        int accumulate, const int* done) {
+                                                        int accumulate, int ncta, const int* done) {
   pdl_enter();
   BAMG_DONE_RETURN
-  const int64_t s = blockIdx.x;
+  const int64_t s = blockIdx.x / ncta;
   const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31, a = wp % BR, sub = wp / BR;
   const int64_t i = srow ? (int64_t)srow[s * 32 + lane] : s * 32 + lane;
-  const T acc = row_component<BR, BC, VS, T, T, T>(sp, col, vals, v, s, lane, a, sub);
+  T acc;
+  if (!row_component<BR, BC, VS, T, T, T>(sp, col, vals, v, s, lane, a, sub, ncta, acc)) return;
   if (sub == 0 && i >= 0 && i < n) y[i * BR + a] = accumulate ? y[i * BR + a] + acc : acc;
 }
 
@@ -371,9 +375,10 @@ static Status smooth_down(bamg_mg* mg, int l, const int* done, cudaStream_t st, 
   for (int k = 0; k < m; ++k) {
     if (BS == 6 && split_for<T>(A)) {
       BAMG_DISPATCH_VS(split_for<T>(A), {
-        BAMG_CUDA(launch_k(k_cheb_step_split<BS, VS, T>, dim3((unsigned)A->nslices), dim3(32 * BS * VS), st, 
+        const int nc = split_cluster(A, VS);
+        BAMG_CUDA(launch_clusters(k_cheb_step_split<BS, VS, T>, dim3((unsigned)A->nslices * nc), dim3(32 * BS * VS), nc, true, st,
             A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, d[k & 1], d[(k + 1) & 1], p.x, p.r, p.dinv, L.weights, sc, k,
-            k + 1 < m ? 1 : 0, done));
+            k + 1 < m ? 1 : 0, nc, done));
         BAMG_COUNT_LAUNCH; })
     } else {
       BAMG_DISPATCH_V(lanes_for<T>(A), { BAMG_CUDA(launch_k(k_cheb_step<BS, V, T>, dim3(gr), dim3(kChebThreads), st, A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, rows, d[k & 1],
@@ -404,8 +409,9 @@ static Status smooth_up(bamg_mg* mg, int l, const int* done, cudaStream_t st, do
   const int pr = prof_begin(mg->ctx, l == 0 ? BAMG_PROF_CHEB_RINIT_L0 : -1, st);
   if (split) {
     BAMG_DISPATCH_VS(split, {
-      BAMG_CUDA(launch_k(k_cheb_rinit_split<BS, VS, T>, dim3(gs), dim3(32 * BS * VS), st, A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, p.x, p.b,
-                                                                 p.r, p.d0, p.dinv, L.weights, sc, done));
+      const int nc = split_cluster(A, VS);
+      BAMG_CUDA(launch_clusters(k_cheb_rinit_split<BS, VS, T>, dim3(gs * nc), dim3(32 * BS * VS), nc, true, st, A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, p.x, p.b,
+                                                                 p.r, p.d0, p.dinv, L.weights, sc, nc, done));
       BAMG_COUNT_LAUNCH; })
   } else {
     BAMG_DISPATCH_V(lanes_for<T>(A), { BAMG_CUDA(launch_k(k_cheb_rinit<BS, V, T>, dim3(gr), dim3(kChebThreads), st, A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, rows, p.x, p.b, p.r,
@@ -419,8 +425,9 @@ static Status smooth_up(bamg_mg* mg, int l, const int* done, cudaStream_t st, do
     if (split) {
       BAMG_DISPATCH_VS(split, {
         auto kern = last ? k_cheb_step_split<BS, VS, T, true> : k_cheb_step_split<BS, VS, T, false>;
-        BAMG_CUDA(launch_k(kern, dim3(gs), dim3(32 * BS * VS), st, A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, d[k & 1],
-                           d[(k + 1) & 1], p.x, p.r, p.dinv, L.weights, sc, k, 1, done));
+        const int nc = split_cluster(A, VS);
+        BAMG_CUDA(launch_clusters(kern, dim3(gs * nc), dim3(32 * BS * VS), nc, true, st, A->slice_ptr, A->sell_col, p.Avals, A->slot_row, L.n, d[k & 1],
+                                  d[(k + 1) & 1], p.x, p.r, p.dinv, L.weights, sc, k, 1, nc, done));
         BAMG_COUNT_LAUNCH; })
     } else {
       BAMG_DISPATCH_V(lanes_for<T>(A), {
@@ -468,8 +475,9 @@ static Status transfer(const bamg_bsr* M, const T* vals, const T* v, T* y, int a
   }
   if (BR == 6 && split_for<T>(M)) {
     BAMG_DISPATCH_VS(split_for<T>(M), {
-      BAMG_CUDA(launch_k(k_transfer_split<BR, BC, VS, T>, dim3((unsigned)M->nslices), dim3(32 * BR * VS), st, M->slice_ptr, M->sell_col, vals,
-                                                                                     M->slot_row, M->nbr, v, y, accumulate, done));
+      const int nc = split_cluster(M, VS);
+      BAMG_CUDA(launch_clusters(k_transfer_split<BR, BC, VS, T>, dim3((unsigned)M->nslices * nc), dim3(32 * BR * VS), nc, true, st,
+                                M->slice_ptr, M->sell_col, vals, M->slot_row, M->nbr, v, y, accumulate, nc, done));
       BAMG_COUNT_LAUNCH; })
     BAMG_CUDA(cudaGetLastError());
     return Status{};

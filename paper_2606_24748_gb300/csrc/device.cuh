@@ -2,6 +2,8 @@
 // the one-thread-per-block-row product, and deterministic reductions.
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include <type_traits>
 
 #include "fixed.cuh"
@@ -138,13 +140,19 @@ __device__ __forceinline__ void row_product(const int* __restrict__ slice_ptr,
 // (one barrier); the result is valid in the sub = 0 warps.  Every thread of
 // the CTA must call this.  The warps read the same column indices and x
 // entries (cached); every value is read once, coalesced.
+// With ncta > 1 a cluster of that many CTAs takes the slice (split_cluster): the
+// chunks are dealt over all their warps, each CTA adds up its own, and the
+// totals meet in CTA 0 through distributed shared memory, in CTA order.  The
+// result is then valid in CTA 0 only; the others return false and are done.
 template <int BR, int BC, int VS, typename TM, typename TA, typename TX>
-__device__ __forceinline__ TA row_component(const int* __restrict__ slice_ptr, const int* __restrict__ col,
-                                            const TM* __restrict__ vals, const TX* __restrict__ x, int64_t s,
-                                            int lane, int a, int sub) {
+__device__ __forceinline__ bool row_component(const int* __restrict__ slice_ptr, const int* __restrict__ col,
+                                              const TM* __restrict__ vals, const TX* __restrict__ x, int64_t s,
+                                              int lane, int a, int sub, int ncta, TA& acc) {
+  namespace cg = cooperative_groups;
+  const int rank = ncta > 1 ? (int)cg::this_cluster().block_rank() : 0;
   const int c0 = __ldg(slice_ptr + s), c1 = __ldg(slice_ptr + s + 1);
-  TA acc = TA(0);
-  for (int c = c0 + sub; c < c1; c += VS) {
+  acc = TA(0);
+  for (int c = c0 + rank * VS + sub; c < c1; c += ncta * VS) {
     const int j = __ldg(col + (int64_t)c * 32 + lane);
     const TM* v = vals + (int64_t)c * (32 * BR * BC) + 32 * (a * BC) + lane;
     TA xv[BC];
@@ -162,7 +170,23 @@ __device__ __forceinline__ TA row_component(const int* __restrict__ slice_ptr, c
       for (int t = 1; t < VS; ++t) acc += part[t][a][lane];
     }
   }
-  return acc;
+  if (ncta > 1) {
+    __shared__ TA total[BR][32];
+    cg::cluster_group cluster = cg::this_cluster();
+    if (sub == 0) total[a][lane] = acc;
+    cluster.sync();
+    if (rank == 0 && sub == 0) {
+      TA far[8];
+#pragma unroll
+      for (int r = 1; r < 8; ++r) far[r] = r < ncta ? *cluster.map_shared_rank(&total[a][lane], r) : TA(0);
+#pragma unroll
+      for (int r = 1; r < 8; ++r)
+        if (r < ncta) acc += far[r];
+    }
+    cluster.sync();  // the other CTAs' totals have been read
+    return rank == 0;
+  }
+  return true;
 }
 
 // Row form of the component split, for matrices with few, very long rows
@@ -558,6 +582,31 @@ inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, cud
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// The same for a kernel whose CTAs work in clusters of `ncta` (1: none).
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_clusters(void (*kernel)(KArgs...), dim3 grid, dim3 block, int ncta, bool dependent,
+                                   cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (dependent) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (ncta > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = (unsigned)ncta;
+    attr[n].val.clusterDim.y = 1;
+    attr[n++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = (unsigned)n;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 

@@ -471,6 +471,19 @@ template <typename T>
 inline int split_for(const bamg_bsr* A) {
   return sizeof(T) == 4 ? A->split32 : A->split;
 }
+// CTAs per slice of the component-split kernels (vs warps per component).  A
+// level with few slices leaves most of the chip idle behind its longest row
+// (MIS hierarchy at 24^3, level 1: 35 slices of up to 100 chunks, y = A x 37 us
+// with 24 warps per slice, 14.7 with a cluster of eight CTAs).  A cluster then
+// shares each slice: as many CTAs as stay resident at once, up to four per SM,
+// with two chunks or more per warp.
+inline int split_cluster(const bamg_bsr* A, int vs) {
+  if (A->nslices <= 0) return 1;
+  const int64_t chunks = A->nchunks / A->nslices, resident = 152 * std::min(4, 2048 / (192 * vs));
+  int n = 1;
+  while (n < 8 && A->nslices * 2 * n <= resident && chunks >= 2LL * (2 * n) * vs) n *= 2;
+  return n;
+}
 // Split codes 32, 64 and 128: the row form (one CTA per row, split / 32 warps
 // per output component).
 constexpr int kSplitRows = 32;

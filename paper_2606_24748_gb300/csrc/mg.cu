@@ -344,13 +344,14 @@ __global__ void __launch_bounds__(768) k_power_step_split(const int* __restrict_
                                                           const double* __restrict__ w_in,
                                                           double* __restrict__ w_out, const double* norm_in,
                                                           double* norm_out, int64_t n, int64_t nslices,
-                                                          double* partials, unsigned* counter) {
+                                                          double* partials, unsigned* counter, int ncta) {
   __shared__ double as[BS][32];
   const double sc = norm_in ? 1.0 / *norm_in : 1.0;
   const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31, a = wp % BS, sub = wp / BS;
   double local[1] = {0.0};
-  for (int64_t s = blockIdx.x; s < nslices; s += gridDim.x) {
-    const double acc = row_component<BS, BS, VS, TM, double, double>(slice_ptr, col, vals, w_in, s, lane, a, sub);
+  for (int64_t s = blockIdx.x / ncta; s < nslices; s += gridDim.x / ncta) {
+    double acc;
+    if (!row_component<BS, BS, VS, TM, double, double>(slice_ptr, col, vals, w_in, s, lane, a, sub, ncta, acc)) continue;
     __syncthreads();  // the previous slice's readers of `as` are done
     if (sub == 0) as[a][lane] = acc * sc;
     __syncthreads();
@@ -449,9 +450,10 @@ static Status power_impl(bamg_mg* mg, const bamg_bsr* A, const TM* vals, const d
     if (split) {
       const unsigned gs = (unsigned)std::max<int64_t>(1, std::min<int64_t>(A->nslices, 1216));
       BAMG_DISPATCH_VS(split, {
-        k_power_step_split<BS, VS, TM><<<gs, 32 * BS * VS, 0, st>>>(A->slice_ptr, A->sell_col, vals, A->slot_row, dinv, wts,
-                                                                     w[it & 1], w[(it + 1) & 1], nin, norms + (it & 1),
-                                                                     n, A->nslices, ctx->d_partials, ctx->d_counters);
+        const int nc = split_cluster(A, VS);
+        BAMG_CUDA(launch_clusters(k_power_step_split<BS, VS, TM>, dim3(nc > 1 ? (unsigned)A->nslices * nc : gs), dim3(32 * BS * VS), nc,
+                                  false, st, A->slice_ptr, A->sell_col, vals, A->slot_row, dinv, wts, w[it & 1],
+                                  w[(it + 1) & 1], nin, norms + (it & 1), n, A->nslices, ctx->d_partials, ctx->d_counters, nc));
         BAMG_COUNT_LAUNCH; })
       continue;
     }

@@ -31,10 +31,12 @@ __global__ void __launch_bounds__(kRowThreads) k_spmv(const int* __restrict__ sl
 template <int BR, int BC, int VS, typename T>
 __global__ void __launch_bounds__(768) k_spmv_split(const int* __restrict__ slice_ptr, const int* __restrict__ col,
                                                     const T* __restrict__ vals, const int* __restrict__ srow,
-                                                    const T* __restrict__ x, T* __restrict__ y, int64_t nbr) {
-  const int64_t s = blockIdx.x;
+                                                    const T* __restrict__ x, T* __restrict__ y, int64_t nbr,
+                                                    int ncta) {
+  const int64_t s = blockIdx.x / ncta;
   const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31, a = wp % BR, sub = wp / BR;
-  const T acc = row_component<BR, BC, VS, T, T, T>(slice_ptr, col, vals, x, s, lane, a, sub);
+  T acc;
+  if (!row_component<BR, BC, VS, T, T, T>(slice_ptr, col, vals, x, s, lane, a, sub, ncta, acc)) return;
   const int64_t i = srow ? (int64_t)srow[s * 32 + lane] : s * 32 + lane;
   if (sub == 0 && i >= 0 && i < nbr) y[i * BR + a] = acc;
 }
@@ -185,12 +187,14 @@ static Status launch_spmv_v(const bamg_bsr* A, int vec, const T* vals, const T* 
   if (vec < 0) {
     if (A->nslices == 0) return Status{};
     BAMG_DISPATCH_VS(-vec, {
+      const int nc = split_cluster(A, VS);
+      const dim3 g((unsigned)A->nslices * nc), t(192 * VS);
       if (A->bc == 6)
-        k_spmv_split<6, 6, VS, T><<<(unsigned)A->nslices, 192 * VS, 0, st>>>(A->slice_ptr, A->sell_col, vals, A->slot_row, x, y,
-                                                                            A->nbr);
+        BAMG_CUDA(launch_clusters(k_spmv_split<6, 6, VS, T>, g, t, nc, false, st, A->slice_ptr, A->sell_col, vals, A->slot_row, x, y,
+                                  A->nbr, nc));
       else
-        k_spmv_split<6, 3, VS, T><<<(unsigned)A->nslices, 192 * VS, 0, st>>>(A->slice_ptr, A->sell_col, vals, A->slot_row, x, y,
-                                                                            A->nbr);
+        BAMG_CUDA(launch_clusters(k_spmv_split<6, 3, VS, T>, g, t, nc, false, st, A->slice_ptr, A->sell_col, vals, A->slot_row, x, y,
+                                  A->nbr, nc));
       BAMG_COUNT_LAUNCH; })
     BAMG_CUDA(cudaGetLastError());
     return Status{};
