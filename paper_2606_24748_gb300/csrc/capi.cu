@@ -273,7 +273,9 @@ Status launch_to_fp32(const double* src, float* dst, int64_t n, cudaStream_t st)
 // time: the values are read as they are stored (32 rows of one element per
 // warp load) and, through shared memory, written as runs of a row's
 // consecutive blocks.  A thread per output value would have each warp load
-// touch 32 lines (64^3 operator: 367 us, of which the bytes take 153).
+// touch 32 lines (64^3 operator: 367 us, of which the bytes take 153).  The
+// loads of a pass are independent, so six are in flight at once: one at a time
+// the kernel waited for each (252 us, 193 with six, 195 with nine, 209 with 18).
 constexpr int kGatherTile = 144;  // values per row and pass
 __host__ __device__ constexpr int gather_chunks(int B) { return B >= kGatherTile ? 1 : kGatherTile / B; }
 
@@ -289,6 +291,7 @@ __global__ void __launch_bounds__(256) k_gather_values(const int* __restrict__ s
   const int c0 = slice_ptr[s], c1 = slice_ptr[s + 1];
   for (int c = c0; c < c1; c += T) {
     const int nc = min(T, c1 - c);
+#pragma unroll 6
     for (int e = warp; e < nc * B; e += nw) tile[lane * pitch + e] = vals[(int64_t)c * 32 * B + 32 * e + lane];
     __syncthreads();
     for (int r = warp; r < 32; r += nw) {
@@ -296,6 +299,7 @@ __global__ void __launch_bounds__(256) k_gather_values(const int* __restrict__ s
       if (row < 0 || row >= nbr) continue;
       const int k0 = rowptr[row] + (c - c0);
       const int n = min(nc, rowptr[row + 1] - k0) * B;  // the row's blocks of this pass
+#pragma unroll 5
       for (int e = lane; e < n; e += 32) out[(int64_t)k0 * B + e] = tile[r * pitch + e];
     }
     __syncthreads();
