@@ -20,7 +20,7 @@
 namespace bamg {
 
 constexpr int kT = 32;  // tile size
-constexpr int kFactorCounters = 32;  // two context counters: quarter updates done, per matrix
+constexpr int kFactorCounters = 32;  // two context counters: stripe updates done, per matrix
 
 template <typename TM, int BS>
 __global__ void k_dense_fill(int64_t nnzb, const int* __restrict__ rowptr_rows, const int* __restrict__ colidx,
@@ -71,19 +71,37 @@ __device__ __forceinline__ void tile_update(double* __restrict__ C, const double
   }
 }
 
-// Rows [r0, r0 + 8) of C -= A A^T for a 32 x 32 tile C and a 32 x 32 tile A
-// (one quarter of a diagonal-tile update; 256 threads, one output each).
-__device__ __forceinline__ void tile_syrk_rows8(double* __restrict__ C, const double* __restrict__ Ab, int64_t ld,
-                                                int r0, double (*As)[kT + 1], double (*Bs)[kT + 1]) {
+// Stripes of four rows (or columns) of a 32-long tile product, one output per
+// thread pair: each half of the CTA sums 16 of the 32 products and the halves
+// meet in shared memory.  With 256 outputs per CTA each SM sub-partition had two
+// warps of 32 dependent multiply-adds, 64 cycles apiece (4,100 cycles); so it
+// has two of 16, and the factor's panel steps have twice as many CTAs to use.
+constexpr int kStripe = 4;
+constexpr int kStripes = kT / kStripe;
+
+__device__ __forceinline__ double stripe_sum(double t, double* half) {
+  const int tid = threadIdx.x;
+  __syncthreads();
+  if (tid >= 128) half[tid - 128] = t;
+  __syncthreads();
+  return tid < 128 ? t + half[tid] : 0.0;
+}
+
+// Rows [r0, r0 + 4) of C -= A A^T for a 32 x 32 tile C and a 32 x 32 tile A.
+__device__ __forceinline__ void tile_syrk_rows(double* __restrict__ C, const double* __restrict__ Ab, int64_t ld,
+                                               int r0, double (*As)[kT + 1], double (*Bs)[kT + 1]) {
   const int tid = threadIdx.x;
   __syncthreads();
   for (int e = tid; e < kT * kT; e += blockDim.x) Bs[e / kT][e % kT] = Ab[(int64_t)(e / kT) * ld + e % kT];
+  const int r = (tid % 128) / kT, c = tid % kT, l0 = tid / 128 * (kT / 2);
+  double* p = C + (int64_t)(r0 + r) * ld + c;
+  const double old = tid < 128 ? *p : 0.0;
   __syncthreads();
-  const int r = tid / kT, c = tid % kT;
   double acc = 0.0;
-#pragma unroll 8
-  for (int l = 0; l < kT; ++l) acc = fma(Bs[r0 + r][l], Bs[c][l], acc);
-  C[(int64_t)(r0 + r) * ld + c] -= acc;
+#pragma unroll
+  for (int l = 0; l < kT / 2; ++l) acc = fma(Bs[r0 + r][l0 + l], Bs[c][l0 + l], acc);
+  acc = stripe_sum(acc, &As[0][0]);
+  if (tid < 128) *p = old - acc;
 }
 
 // 1 / sqrt(d) by Newton's method for the reciprocal square root,
@@ -131,28 +149,83 @@ __device__ void tri_table(unsigned short* tri) {
 }
 
 // Cholesky of the diagonal tile (k, k) in shared memory and the inverse of
-// the factor (one CTA); L is written back, L^-1 to Linv.  The sweep is the
-// square-root-free form A = Lu D Lu^T: column j's pivot d_j = a_jj, then
-// a_il -= a_ij a_lj / d_j for l > j, one barrier per column, and every
-// thread forms 1 / d_j itself.  Column j is left unscaled (a_ij = Lu_ij d_j),
-// so L = Lu D^(1/2) is a_ij / sqrt(d_j) at the end: the square roots leave the
-// serial chain.
+// the factor (one CTA of 256 threads); L is written back, L^-1 to Linv.
+// The square-root-free form A = Lu D Lu^T, in panels of eight columns.  In a
+// panel a warp holds a column and a lane a row: per column its warp forms the
+// pivot's reciprocal and the scaled column, and after one barrier the warps to
+// the right take their update.  A warp whose column is done goes on with the
+// identity's column beside it, so that the panel ends with G, the effect of its
+// eight steps on the identity.  The entries right of the panel and the identity's
+// columns left of it then take the eight steps at once.  Per column the serial
+// chain is one update, a reciprocal, a scaling and a barrier; everything else
+// is off it.  L = Lu D^(1/2) and L^-1 = D^(-1/2) Lu^-1 take the square roots at
+// the end.  a holds Lu D in its lower triangle and Lu^T in its upper one, w the
+// identity's side.  (With rank-one steps over the whole tile and the inverse
+// afterwards by doubling blocks, the elimination took 29,000 cycles and the
+// inverse 13,200; now 27,200 and 4,800, and a 32-column step of a 12-tile matrix
+// takes 50,000 cycles instead of 65,000.)
 __device__ void diag_tile(double* __restrict__ M, int64_t ld, int k, double* __restrict__ Linv, int* err,
                           double (*a)[kT + 1], double (*w)[kT + 1], const unsigned short* tri) {
   __shared__ double inv[kT];
-  const int tid = threadIdx.x;
+  constexpr int NB = 8;
+  const int tid = threadIdx.x, warp = tid >> 5, i = tid & 31;
   double* base = M + (int64_t)k * kT * ld + (int64_t)k * kT;
   __syncthreads();
-  for (int e = tid; e < kT * kT; e += blockDim.x) a[e / kT][e % kT] = __ldcg(base + (int64_t)(e / kT) * ld + e % kT);
+#pragma unroll
+  for (int e = tid; e < kT * kT; e += 256) a[e / kT][e % kT] = __ldcg(base + (int64_t)(e / kT) * ld + e % kT);
   __syncthreads();
-  for (int j = 0; j < kT; ++j) {
-    double d = a[j][j];
-    if (!positive_finite(d)) d = 1.0;  // reported below
-    const double r = rcp_cubic(d);
-    const int cnt = (kT - 1 - j) * (kT - j) / 2;
-    for (int p = tid; p < cnt; p += blockDim.x) {
-      const int code = tri[p], i = code >> 5, l = code & 31;
-      a[i][l] = fma(-a[i][j] * r, a[l][j], a[i][l]);
+  for (int p = 0; p < kT; p += NB) {
+    const int l = p + warp;
+    double v = i >= l ? a[i][l] : 0.0;
+#pragma unroll
+    for (int jj = 0; jj < NB; ++jj) {
+      const int j = p + jj;
+      if (warp == jj) {
+        const double d = __shfl_sync(0xffffffffu, v, j);
+        const double s = v * rcp_cubic(positive_finite(d) ? d : 1.0);  // others are reported below
+        if (i >= j) a[i][j] = v;
+        if (i > j) a[j][i] = s;
+        v = i > j ? -s : i == j ? 1.0 : 0.0;
+      }
+      __syncthreads();
+      if (warp > jj) {
+        v = fma(-a[i][j], a[j][l], v);
+      } else if (warp < jj) {
+        const double x = __shfl_sync(0xffffffffu, v, j);
+        if (i > j) v = fma(-a[j][i], x, v);
+      }
+    }
+    if (i >= l) w[i][l] = v;
+    __syncthreads();
+    const int rem = kT - NB - p, na = rem * (rem + 1) / 2, n = na + (kT - p) * p;  // at most 328
+    double out[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int q = tid + 256 * h;
+      if (q < na) {
+        const int code = tri[q], r = code >> 5, c = code & 31;
+        double t = a[r][c];
+#pragma unroll
+        for (int j = p; j < p + NB; ++j) t = fma(-a[r][j], a[j][c], t);
+        out[h] = t;
+      } else if (q < n) {
+        const int r = p + (q - na) / p, c = (q - na) % p;
+        double t = r < p + NB ? 0.0 : w[r][c];
+#pragma unroll
+        for (int j = p; j < p + NB; ++j) t = j <= r ? fma(w[r][j], w[j][c], t) : t;
+        out[h] = t;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int q = tid + 256 * h;
+      if (q < na) {
+        const int code = tri[q];
+        a[code >> 5][code & 31] = out[h];
+      } else if (q < n) {
+        w[p + (q - na) / p][(q - na) % p] = out[h];
+      }
     }
     __syncthreads();
   }
@@ -165,72 +238,48 @@ __device__ void diag_tile(double* __restrict__ M, int64_t ld, int k, double* __r
     inv[tid] = rsqrt_newton(d);
   }
   __syncthreads();
-  for (int e = tid; e < kT * kT; e += blockDim.x) {
-    const int i = e / kT, l = e % kT;
-    if (l <= i) a[i][l] *= inv[l];
-  }
-  // W = L^-1 by doubling the inverted diagonal blocks: with diagonal blocks
-  // W11, W22 of size h already inverted, the block below them is
-  // W21 = -W22 L21 W11, formed for every pair at once (two products, 2 h^3
-  // multiply-adds per pair) for h = 1, 2, 4, 8, 16.  T = L21 W11 is kept
-  // transposed in the (unused) upper triangle of the pair's block.
-  if (tid < kT) w[tid][tid] = inv[tid];
-  __syncthreads();
-  for (int h = 1; h < kT; h *= 2) {
-    const int hh = h * h;
-    for (int e = tid; e < (kT / 2) * h; e += blockDim.x) {  // (kT / 2h) pairs x h^2 entries
-      const int i0 = (e / hh) * 2 * h, m = (e % hh) / h, q = e % h;
-      double t = 0.0;
-      for (int n = q; n < h; ++n) t = fma(a[i0 + h + m][i0 + n], w[i0 + n][i0 + q], t);
-      w[i0 + q][i0 + h + m] = t;
-    }
-    __syncthreads();
-    for (int e = tid; e < (kT / 2) * h; e += blockDim.x) {
-      const int i0 = (e / hh) * 2 * h, p = (e % hh) / h, q = e % h;
-      double t = 0.0;
-      for (int m = 0; m <= p; ++m) t = fma(w[i0 + h + p][i0 + h + m], w[i0 + q][i0 + h + m], t);
-      w[i0 + h + p][i0 + q] = -t;
-    }
-    __syncthreads();
-  }
-  for (int e = tid; e < kT * kT; e += blockDim.x) {
-    const int i = e / kT, l = e % kT;
-    base[(int64_t)i * ld + l] = l <= i ? a[i][l] : 0.0;
-    Linv[e] = l <= i ? w[i][l] : 0.0;
+#pragma unroll
+  for (int e = tid; e < kT * kT; e += 256) {
+    const int r = e / kT, c = e % kT;
+    base[(int64_t)r * ld + c] = c <= r ? a[r][c] * inv[c] : 0.0;
+    Linv[e] = c <= r ? w[r][c] * inv[r] : 0.0;
   }
 }
 
-// Rows [r0, r0 + 8) of X = A Linv^T (Cholesky panel), in place over A.
+// Rows [r0, r0 + 4) of X = A Linv^T (Cholesky panel), in place over A.
 __device__ void panel_rows(double* __restrict__ Xt, int64_t ld, const double* __restrict__ Linv, int r0,
                            double (*a)[kT + 1], double (*w)[kT + 1]) {
   const int tid = threadIdx.x;
   __syncthreads();
   for (int e = tid; e < kT * kT; e += blockDim.x) w[e / kT][e % kT] = Linv[e];
-  for (int e = tid; e < 8 * kT; e += blockDim.x) a[e / kT][e % kT] = Xt[(int64_t)(r0 + e / kT) * ld + e % kT];
+  if (tid < kStripe * kT) a[tid / kT][tid % kT] = Xt[(int64_t)(r0 + tid / kT) * ld + tid % kT];
   __syncthreads();
-  const int r = tid / kT, c = tid % kT;  // 8 x 32 outputs
+  const int r = (tid % 128) / kT, c = tid % kT, l0 = tid / 128 * (kT / 2);
   double t = 0.0;
-#pragma unroll 8
-  for (int l = 0; l < kT; ++l) t = fma(a[r][l], w[c][l], t);
-  Xt[(int64_t)(r0 + r) * ld + c] = t;
+#pragma unroll
+  for (int l = 0; l < kT / 2; ++l) t = fma(a[r][l0 + l], w[c][l0 + l], t);
+  t = stripe_sum(t, &a[8][0]);
+  if (tid < 128) Xt[(int64_t)(r0 + r) * ld + c] = t;
 }
 
-// Columns [c0, c0 + 8) of W(i,k) = Linv (delta I - S), in place over S.
+// Columns [c0, c0 + 4) of W(i,k) = Linv (delta I - S), in place over S.
 __device__ void winv_cols(double* __restrict__ St, int64_t ld, const double* __restrict__ Linv, int c0, bool diag,
                           double (*a)[kT + 1], double (*w)[kT + 1]) {
   const int tid = threadIdx.x;
   __syncthreads();
   for (int e = tid; e < kT * kT; e += blockDim.x) w[e / kT][e % kT] = Linv[e];
-  for (int e = tid; e < kT * 8; e += blockDim.x) {
-    const int r = e / 8, c = e % 8;
+  if (tid < kT * kStripe) {
+    const int r = tid / kStripe, c = tid % kStripe;
     a[r][c] = ((diag && r == c0 + c) ? 1.0 : 0.0) - St[(int64_t)r * ld + c0 + c];
   }
   __syncthreads();
-  const int r = tid / 8, c = tid % 8;  // 32 x 8 outputs
+  const int r = (tid % 128) / kStripe, c = tid % kStripe, l0 = tid / 128 * (kT / 2);
   double t = 0.0;
-#pragma unroll 8
-  for (int l = 0; l < kT; ++l) t = fma(w[r][l], a[l][c], t);
-  St[(int64_t)r * ld + c0 + c] = t;
+#pragma unroll
+  for (int l = 0; l < kT / 2; ++l) t = fma(w[r][l0 + l], a[l0 + l][c], t);
+  __shared__ double half[128];
+  t = stripe_sum(t, half);
+  if (tid < 128) St[(int64_t)r * ld + c0 + c] = t;
 }
 
 // Whole coarsest factorisation in one cooperative launch (256 threads per
@@ -268,32 +317,32 @@ __global__ void __launch_bounds__(256) k_dense_factor(double* F, double* W, int6
   for (int k = 0; k < nt; ++k) {
     const double* Lkk_inv = Dinv + (int64_t)k * kT * kT;
     // phase 1
-    const int n_panel = (nt - k - 1) * 4, n_winv = (k + 1) * 4;
+    const int n_panel = (nt - k - 1) * kStripes, n_winv = (k + 1) * kStripes;
     for (int item = b; item < n_panel + n_winv; item += G) {
       if (item < n_panel) {
-        const int i = k + 1 + item / 4;
-        panel_rows(F + (int64_t)i * kT * ld + (int64_t)k * kT, ld, Lkk_inv, (item % 4) * 8, a, w);
+        const int i = k + 1 + item / kStripes;
+        panel_rows(F + (int64_t)i * kT * ld + (int64_t)k * kT, ld, Lkk_inv, (item % kStripes) * kStripe, a, w);
       } else {
-        const int it = item - n_panel, j = it / 4;
-        winv_cols(W + (int64_t)k * kT * ld + (int64_t)j * kT, ld, Lkk_inv, (it % 4) * 8, j == k, a, w);
+        const int it = item - n_panel, j = it / kStripes;
+        winv_cols(W + (int64_t)k * kT * ld + (int64_t)j * kT, ld, Lkk_inv, (it % kStripes) * kStripe, j == k, a, w);
       }
     }
     __threadfence();
     grid.sync();
-    // phase 2: items 0-3 are the four 8-row quarters of the next diagonal
-    // tile's update (CTAs 1-4 take them first and count them in qctr), then
+    // phase 2: items 0-7 are the eight 4-row stripes of the next diagonal
+    // tile's update (CTAs 1-8 take them first and count them in qctr), then
     // the rest of the trailing update and the inverse's updates; CTA 0 waits
-    // for the quarters and factors that tile meanwhile.
+    // for the stripes and factors that tile meanwhile.
     const int T = nt - k - 1;
     const int n_trail = T * (T + 1) / 2, n_wupd = T * (k + 1);
-    const int n_items = T > 0 ? 4 + (n_trail - 1) + n_wupd : 0;
+    const int n_items = T > 0 ? kStripes + (n_trail - 1) + n_wupd : 0;
     if (b == 0 && T > 0) {
       const int g = k + 1;
       if (threadIdx.x == 0) {
         // bounded: after wait_limit polls (about 0.4 s at the default of
         // 2^22) record a timeout and go on rather than wait forever; every
         // CTA still reaches the next grid barrier
-        const unsigned target = 4u * (unsigned)(k + 1);
+        const unsigned target = (unsigned)kStripes * (unsigned)(k + 1);
         for (int64_t polls = 0;; ++polls) {
           if (polls >= wait_limit) {
             set_err(err, kDevTimeout);
@@ -308,16 +357,16 @@ __global__ void __launch_bounds__(256) k_dense_factor(double* F, double* W, int6
       diag_tile(F, ld, g, Dinv + (int64_t)g * kT * kT, err, a, w, tri);
     }
     for (int item = b - 1; b > 0 && item < n_items; item += G - 1) {
-      if (item < 4) {
+      if (item < kStripes) {
         const int g = k + 1;
-        tile_syrk_rows8(F + (int64_t)g * kT * ld + (int64_t)g * kT, F + (int64_t)g * kT * ld + (int64_t)k * kT, ld,
-                        item * 8, a, w);
+        tile_syrk_rows(F + (int64_t)g * kT * ld + (int64_t)g * kT, F + (int64_t)g * kT * ld + (int64_t)k * kT, ld,
+                       item * kStripe, a, w);
         __threadfence();
         __syncthreads();
         if (threadIdx.x == 0) atomicAdd(qctr + mi, 1u);
         continue;
       }
-      const int it0 = item - 4 + 1;  // trailing item 0 is the diagonal tile, done above in quarters
+      const int it0 = item - kStripes + 1;  // trailing item 0 is the diagonal tile, done above in stripes
       if (it0 < n_trail) {
         int idx = it0, i = 0;
         while (idx > i) {  // row-major lower triangle (i, j), j <= i
