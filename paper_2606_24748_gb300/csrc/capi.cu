@@ -148,7 +148,7 @@ Status bsr_set_pattern(bamg_bsr* A, std::vector<int>&& rowptr, std::vector<int>&
   A->nnzb = rowptr[nbr];
   A->nslices = (nbr + kSlice - 1) / kSlice;
   // row of each row position (identity, or sorted by decreasing length within
-  // windows of 1,024 rows; padding positions past nbr stay at the end)
+  // windows of 1,024 rows, and then by slices; padding positions hold -1)
   std::vector<int> order((size_t)A->nslices * kSlice);
   for (size_t r = 0; r < order.size(); ++r) order[r] = (int64_t)r < nbr ? (int)r : -1;
   auto len = [&](int i) { return i < 0 ? -1 : rowptr[i + 1] - rowptr[i]; };
@@ -172,7 +172,21 @@ Status bsr_set_pattern(bamg_bsr* A, std::vector<int>&& rowptr, std::vector<int>&
     // (rows of very uneven length, e.g. Q2 vertex and mid-edge nodes); evenly
     // filled slices keep the identity order and its contiguous vectors
     if (sort_rows == kSortAlways || 10 * stored_chunks(sorted) <= 9 * stored_chunks(order)) {
-      order = std::move(sorted);
+      // Slices in order of decreasing width over the whole matrix.  CTAs go to
+      // the SMs in turn, and with the windows one after another (32 slices
+      // each, wide to narrow) an SM's CTAs came from the same few places of
+      // every window: its work was up to 1.3 times another's, with about one
+      // wave of CTAs nothing evened that out, and a wide slice could come last
+      // (21^3 Q2 elements: SMs busy 62,000 to 100,000 cycles).  Wide to narrow,
+      // each SM gets a like share of every width: FP32 product 50.7 to 47.1 us,
+      // FP64 84.6 to 74.4, a whole 16^3 Q2 step 17.5 to 15.3 ms; the assembly
+      // gains too (345 to 322 us).  A row's sum does not depend on its place.
+      std::vector<int64_t> by((size_t)A->nslices);
+      for (size_t q = 0; q < by.size(); ++q) by[q] = (int64_t)q;
+      auto width = [&](int64_t q) { return len(sorted[(size_t)q * kSlice]); };
+      std::stable_sort(by.begin(), by.end(), [&](int64_t a, int64_t b) { return width(a) > width(b); });
+      for (size_t q = 0; q < by.size(); ++q)
+        std::copy_n(sorted.begin() + by[q] * kSlice, kSlice, order.begin() + q * kSlice);
     } else {
       sort_rows = kSortNever;
     }

@@ -396,8 +396,9 @@ void prof_harvest(bamg_ctx* ctx, std::vector<ProfPair>& pairs, size_t count, int
 // allocates zeroed values.  Used by COO preallocation and the Galerkin symbolic.
 // sort_rows: place the rows in the slices by decreasing length within
 // windows of 1,024 rows (sliced ELL with sorting), so that rows of equal
-// length share slices and little padding is stored; kernels then map each
-// row position to its row through slot_row.
+// length share slices and little padding is stored, the slices themselves by
+// decreasing width; kernels then map each row position to its row through
+// slot_row.
 // Row order of the sliced storage: identity, rows sorted by decreasing length
 // within windows of 1,024 rows (slot_row maps positions to rows), or sorted
 // only where that removes at least a tenth of the stored slots.
