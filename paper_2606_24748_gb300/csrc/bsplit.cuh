@@ -31,23 +31,23 @@ __device__ __forceinline__ void row_blocks_split(const int* __restrict__ slice_p
     row_sums_fx<BR, BC, VB>(c0 + w, c1, col, vals, x, lane, acc);
   } else {
 #pragma unroll
-  for (int r = 0; r < BR; ++r) acc[r] = TA(0);
-  for (int c = c0 + w; c < c1; c += VB) {
-    const int j = __ldg(col + (int64_t)c * 32 + lane);
-    const TM* v = vals + (int64_t)c * (32 * BR * BC) + lane;
-    // the block's values are all requested before the gather of x, so that
-    // their loads are in flight together
-    TM blk[BR * BC];
+    for (int r = 0; r < BR; ++r) acc[r] = TA(0);
+    for (int c = c0 + w; c < c1; c += VB) {
+      const int j = __ldg(col + (int64_t)c * 32 + lane);
+      const TM* v = vals + (int64_t)c * (32 * BR * BC) + lane;
+      // the block's values are all requested before the gather of x, so that
+      // their loads are in flight together
+      TM blk[BR * BC];
 #pragma unroll
-    for (int e = 0; e < BR * BC; ++e) blk[e] = __ldcs(v + 32 * e);
-    TA xv[BC];
+      for (int e = 0; e < BR * BC; ++e) blk[e] = __ldcs(v + 32 * e);
+      TA xv[BC];
 #pragma unroll
-    for (int q = 0; q < BC; ++q) xv[q] = (TA)__ldg(x + (int64_t)j * BC + q);
+      for (int q = 0; q < BC; ++q) xv[q] = (TA)__ldg(x + (int64_t)j * BC + q);
 #pragma unroll
-    for (int r = 0; r < BR; ++r)
+      for (int r = 0; r < BR; ++r)
 #pragma unroll
-      for (int q = 0; q < BC; ++q) acc[r] = fma((TA)blk[r * BC + q], xv[q], acc[r]);
-  }
+        for (int q = 0; q < BC; ++q) acc[r] = fma((TA)blk[r * BC + q], xv[q], acc[r]);
+    }
   }
   __shared__ TA part[VB][BR][32];
 #pragma unroll

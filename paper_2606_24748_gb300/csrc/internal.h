@@ -176,7 +176,7 @@ struct bamg_ptap {
   int *s2_slot = nullptr, *s2_tslot = nullptr, *s2_off = nullptr, *s2_p = nullptr, *s2_z = nullptr;
   int rounds1 = 1;  // stage 1: rounds of items per CTA
   // work buffers and the state-gated prolongator-side cache (P in block order)
-  double* Z = nullptr;
+  double* Z = nullptr;  // FP64 products' intermediate; lent to FP32 ones (see ptap_run)
   float* Z32 = nullptr;
   double* Pblk = nullptr;
   float* Pblk32 = nullptr;

@@ -6,10 +6,14 @@
 // its column over the block pairs (A_ik, P_kJ) in the output's gather list.
 // Stage 2 computes A_c = P^T Z the same way over the pairs (P_iI, Z_iJ).
 // Lists are fixed by the symbolic phase, so results are deterministic and no
-// atomics are used.  With FP64 arithmetic at 2 FMA/clock/SM the kernels are
-// bound by the FP64 pipe, not by memory; the gather lists keep every FMA
-// useful (no padding to dense local blocks) and the work-sorted item order
-// keeps the lane groups of a warp busy for the same number of steps.
+// atomics are used.  The gather lists keep every FMA useful (no padding to dense
+// local blocks).  The FP64 pipe, at 2 FMA/clock/SM, would take 4.0 ms for the
+// finest level's product at 64^3; a third of the rows runs there and the rest
+// in block-scaled fixed point on the integer pipes (fixed.cuh), from operands
+// cut once per block instead of once per pair (64^3: stage 1 2.86 -> 1.70 ms
+// with the cut, stage 2 1.21 -> 0.63).  Stage 1 takes its items in runs of a
+// row, so that a warp's lane groups share the row's A blocks; stage 2 in
+// windows ordered by work, a long list shared by up to eight warps.
 #include <algorithm>
 #include <numeric>
 
@@ -714,17 +718,16 @@ static Status cut_operator(bamg_ptap* pl, const bamg_bsr* A) {
 }
 
 // FP32 copy of A's blocks for this product, padded.
-static Status pad_operator(bamg_ptap* pl, const bamg_bsr* A) {
+static Status pad_operator(bamg_ptap* pl, const bamg_bsr* A, float* Apad) {
   cudaStream_t st = pl->ctx->stream;
   const int64_t n = A->nslots();
   if (n == 0) return Status{};
-  if (!pl->Apad) BAMG_TRY(dalloc(&pl->Apad, n * block_pitch<float>(pl->bs * pl->bs), st));
   const unsigned b = (unsigned)((n + 127) / 128);
   const int pm = prof_begin(pl->ctx, pl->prof_stage1, st, 0);
   if (pl->bs == 6)
-    k_pad_slots<6><<<b, 128, 0, st>>>(n, A->vals32, (float4*)pl->Apad);
+    k_pad_slots<6><<<b, 128, 0, st>>>(n, A->vals32, (float4*)Apad);
   else
-    k_pad_slots<3><<<b, 128, 0, st>>>(n, A->vals32, (float4*)pl->Apad);
+    k_pad_slots<3><<<b, 128, 0, st>>>(n, A->vals32, (float4*)Apad);
   BAMG_COUNT_LAUNCH;
   prof_end(pl->ctx, pm, st);
   BAMG_CUDA(cudaGetLastError());
@@ -751,12 +754,21 @@ Status ptap_run(bamg_ptap* pl, bamg_bsr* A, bamg_bsr* P, bamg_bsr* Ac, bamg_prec
   } else if (prec == BAMG_FP32) {
     BAMG_TRY(bsr_ensure_fp32(A));
     BAMG_TRY(refresh_pblk(pl, P, true));
-    if (!pl->Z32) BAMG_TRY(dalloc(&pl->Z32, pl->nz * pl->bs * pl->bsp, st));
     if (stage2 && !Ac->vals32) BAMG_TRY(dalloc(&Ac->vals32, Ac->nslots() * Ac->block_elems(), st));
     if (stage2 && Ac->vals32 && Ac->vals32_version == ~0ull)
       BAMG_CUDA(cudaMemsetAsync(Ac->vals32, 0, sizeof(float) * Ac->nslots() * Ac->block_elems(), st));
-    BAMG_TRY(pad_operator(pl, A));
-    BAMG_TRY(run_stages<float>(pl, pl->Apad, pl->Pblk32, pl->Z32, stage2 ? Ac->vals32 : nullptr, stage2));
+    // The FP64 intermediate's memory, scratch of the other precision, holds A's
+    // padded copy where that fits (3x3 blocks), or else the FP32 intermediate;
+    // the other one is allocated by the first FP32 product (47^3: with both
+    // allocated that product took 1,190 us, so 1,035).
+    const int64_t na = A->nslots() * block_pitch<float>(pl->bs * pl->bs), nz = pl->nz * pl->bs * pl->bsp;
+    const bool pad_in_z = na <= 2 * nz;
+    if (pad_in_z && !pl->Z32) BAMG_TRY(dalloc(&pl->Z32, nz, st));
+    if (!pad_in_z && !pl->Apad) BAMG_TRY(dalloc(&pl->Apad, na, st));
+    float* Apad = pad_in_z ? reinterpret_cast<float*>(pl->Z) : pl->Apad;
+    float* Z32 = pad_in_z ? pl->Z32 : reinterpret_cast<float*>(pl->Z);
+    BAMG_TRY(pad_operator(pl, A, Apad));
+    BAMG_TRY(run_stages<float>(pl, Apad, pl->Pblk32, Z32, stage2 ? Ac->vals32 : nullptr, stage2));
     if (stage2) {
       Ac->version++;
       Ac->vals32_version = Ac->version;
