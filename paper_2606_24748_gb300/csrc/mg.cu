@@ -438,7 +438,6 @@ template <int BS, typename TM>
 static Status power_impl(bamg_mg* mg, const bamg_bsr* A, const TM* vals, const double* dinv, const float* wts,
                          bool scalar_diag, double* out_scal, cudaStream_t st) {
   bamg_ctx* ctx = mg->ctx;
-  
   const int64_t n = A->nbr, rows = row_threads_for<TM>(A);
   double* w[2] = {mg->power_w[0], mg->power_w[1]};
   double* norms = mg->scal + (int64_t)mg->levels.size() * kScalarsPerLevel;  // 2 scratch slots
