@@ -147,50 +147,9 @@ Status bsr_set_pattern(bamg_bsr* A, std::vector<int>&& rowptr, std::vector<int>&
   if ((int64_t)rowptr.size() != nbr + 1) return make_status(BAMG_ERR_INVALID, "rowptr size");
   A->nnzb = rowptr[nbr];
   A->nslices = (nbr + kSlice - 1) / kSlice;
-  // row of each row position (identity, or sorted by decreasing length within
-  // windows of 1,024 rows, and then by slices; padding positions hold -1)
-  std::vector<int> order((size_t)A->nslices * kSlice);
-  for (size_t r = 0; r < order.size(); ++r) order[r] = (int64_t)r < nbr ? (int)r : -1;
+  const Placement placed = place_rows(rowptr, nbr, sort_rows);
+  const std::vector<int>& order = placed.order;
   auto len = [&](int i) { return i < 0 ? -1 : rowptr[i + 1] - rowptr[i]; };
-  auto stored_chunks = [&](const std::vector<int>& ord) {
-    int64_t c = 0;
-    for (int64_t s = 0; s < A->nslices; ++s) {
-      int w = 0;
-      for (int64_t r = s * kSlice; r < (s + 1) * kSlice; ++r) w = std::max(w, len(ord[r]));
-      c += w;
-    }
-    return c;
-  };
-  if (sort_rows != kSortNever) {
-    std::vector<int> sorted = order;
-    constexpr size_t kWindow = 1024;
-    for (size_t w0 = 0; w0 < sorted.size(); w0 += kWindow) {
-      const size_t w1 = std::min(sorted.size(), w0 + kWindow);
-      std::stable_sort(sorted.begin() + w0, sorted.begin() + w1, [&](int a, int b) { return len(a) > len(b); });
-    }
-    // auto: only where the sort removes a tenth of the stored slots or more
-    // (rows of very uneven length, e.g. Q2 vertex and mid-edge nodes); evenly
-    // filled slices keep the identity order and its contiguous vectors
-    if (sort_rows == kSortAlways || 10 * stored_chunks(sorted) <= 9 * stored_chunks(order)) {
-      // Slices in order of decreasing width over the whole matrix.  CTAs go to
-      // the SMs in turn, and with the windows one after another (32 slices
-      // each, wide to narrow) an SM's CTAs came from the same few places of
-      // every window: its work was up to 1.3 times another's, with about one
-      // wave of CTAs nothing evened that out, and a wide slice could come last
-      // (21^3 Q2 elements: SMs busy 62,000 to 100,000 cycles).  Wide to narrow,
-      // each SM gets a like share of every width: FP32 product 50.7 to 47.1 us,
-      // FP64 84.6 to 74.4, a whole 16^3 Q2 step 17.5 to 15.3 ms; the assembly
-      // gains too (345 to 322 us).  A row's sum does not depend on its place.
-      std::vector<int64_t> by((size_t)A->nslices);
-      for (size_t q = 0; q < by.size(); ++q) by[q] = (int64_t)q;
-      auto width = [&](int64_t q) { return len(sorted[(size_t)q * kSlice]); };
-      std::stable_sort(by.begin(), by.end(), [&](int64_t a, int64_t b) { return width(a) > width(b); });
-      for (size_t q = 0; q < by.size(); ++q)
-        std::copy_n(sorted.begin() + by[q] * kSlice, kSlice, order.begin() + q * kSlice);
-    } else {
-      sort_rows = kSortNever;
-    }
-  }
   std::vector<int> sp(A->nslices + 1, 0);
   for (int64_t s = 0; s < A->nslices; ++s) {
     int w = 0;
@@ -235,7 +194,7 @@ Status bsr_set_pattern(bamg_bsr* A, std::vector<int>&& rowptr, std::vector<int>&
   dfree(A->slot_row, st);
   dfree(A->vals, st);
   dfree(A->vals32, st);
-  if (sort_rows != kSortNever) BAMG_TRY(upload(&A->slot_row, order, st));
+  if (placed.sorted) BAMG_TRY(upload(&A->slot_row, order, st));
   BAMG_TRY(upload(&A->rowptr, A->h_rowptr, st));
   BAMG_TRY(upload(&A->colidx, A->h_colidx, st));
   BAMG_TRY(upload(&A->slice_ptr, sp, st));

@@ -232,7 +232,7 @@ __device__ __forceinline__ void row_of_thread(int64_t t, int64_t& row, int& sub)
 }
 
 // Block row stored at row position pos.  Slices sorted by row length carry
-// the map (srow; -1 at the padding positions past the last row); otherwise
+// the map (srow; -1 at the padding positions, which are the last ones); otherwise
 // the position is the row.  Vectors and block-diagonal inverses stay indexed
 // by row in either case.
 __device__ __forceinline__ int64_t row_at(const int* __restrict__ srow, int64_t pos) {

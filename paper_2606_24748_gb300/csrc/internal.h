@@ -11,11 +11,10 @@
 #include <vector>
 
 #include "bamg.h"
+#include "placement.h"
 
 namespace bamg {
 
-// Rows per slice of the sliced block storage: one warp, one row per lane.
-constexpr int kSlice = 32;
 // Threads per CTA of the row kernels (4 slices).
 constexpr int kRowThreads = 128;
 // CTAs of the fixed-grid reductions (a multiple of the 152 SMs of a GB300).
@@ -126,7 +125,8 @@ struct bamg_bsr {
   int* slot_of = nullptr;    // nnzb: CSR block -> slot
   int* diag_slot = nullptr;  // nbr (square blocks only, -1 if no diagonal block)
   int* slot_row = nullptr;   // sorted slices: block row of each of the 32 * nslices row positions
-                             // (-1 = padding); null when row position = row
+                             // (-1 = padding, at positions nbr and up only: see placement.h); null
+                             // when row position = row
   bool all_diag = false;     // every block row has its diagonal block
   int vec = 1;               // lanes per block row of the FP64 row kernels (1..32, power of 2)
   int vec32 = 1;             // the same for kernels reading the FP32 copy
@@ -394,15 +394,8 @@ void prof_harvest(bamg_ctx* ctx, std::vector<ProfPair>& pairs, size_t count, int
 // ------------------------------------------------------------ pattern helpers
 // Build the sliced form (and device/host CSR copies) from a host CSR pattern;
 // allocates zeroed values.  Used by COO preallocation and the Galerkin symbolic.
-// sort_rows: place the rows in the slices by decreasing length within
-// windows of 1,024 rows (sliced ELL with sorting), so that rows of equal
-// length share slices and little padding is stored, the slices themselves by
-// decreasing width; kernels then map each row position to its row through
-// slot_row.
-// Row order of the sliced storage: identity, rows sorted by decreasing length
-// within windows of 1,024 rows (slot_row maps positions to rows), or sorted
-// only where that removes at least a tenth of the stored slots.
-constexpr int kSortNever = 0, kSortAlways = 1, kSortAuto = 2;
+// sort_rows: the row order of the slices (placement.h); kernels map each row
+// position of a sorted matrix to its row through slot_row.
 Status bsr_set_pattern(bamg_bsr* A, std::vector<int>&& rowptr, std::vector<int>&& colidx, int sort_rows = kSortNever);
 Status bsr_ensure_fp32(bamg_bsr* A);   // refresh vals32 if the version changed
 void bsr_release(bamg_bsr* A);
