@@ -220,9 +220,10 @@ BAMG_API bamg_status bamg_bsr_spmm(bamg_bsr* A, const void* X, void* Y, int k, b
  * flushed L2 on the context's stream and keeps the fastest (a choice must
  * beat the best one before it by 3%, against timing noise), for the FP64
  * values and, when present, the FP32 copy (allocates work vectors; returns
- * the FP64 choice and its time in ms, either may be NULL).  Results do not
- * depend on the choice beyond summation order.  _set_lanes applies to both
- * copies. */
+ * the FP64 choice and its time in ms, either may be NULL).  Choices differ by
+ * rounding alone: with any of them every entry of an FP64 product, and of
+ * those inside the cycle and the Galerkin products, is within n 2^-52 of its
+ * own sum of |a| |x| over its n terms.  _set_lanes applies to both copies. */
 BAMG_API bamg_status bamg_bsr_autotune(bamg_bsr* A, int* lanes, float* ms);
 BAMG_API bamg_status bamg_bsr_set_lanes(bamg_bsr* A, int lanes);
 BAMG_API bamg_status bamg_bsr_get_lanes(const bamg_bsr* A, int* lanes);
@@ -478,8 +479,8 @@ BAMG_API bamg_status bamg_cg_solve(bamg_mg* mg, const double* b, double* x, doub
  * bamg_mg_vcycle_multi: X = M B, one V-cycle per column from x = 0.  Per
  * column the arithmetic and its order are those of bamg_vcycle with one lane
  * per block row on every operator (bamg_bsr_set_lanes(.., 1)), so the
- * results then agree bit for bit; with other lane counts they differ only by
- * summation order.
+ * results then agree bit for bit; with other lane counts they differ by
+ * rounding.
  *
  * bamg_cg_solve_multi: k independent preconditioned CG recurrences (the
  * iterates of bamg_cg_solve on each column, up to the summation order of the

@@ -35,9 +35,10 @@ __device__ __forceinline__ double warp_sum(double v) {
 // through the read-only path, where neighbouring rows hit the same lines.
 // `row` is the thread's row; `sub` its lane within the row's group.
 // FP64 products of 3x3 and 3x6 blocks (the finest operator and prolongator)
-// are formed on the FP64 and the integer pipes together (fixed.cuh): the FP64 pipe alone bounds the
-// 64^3 operator (7.19 M blocks) at 107 us, HBM at 81.  Measured there: y = A x
-// 128 -> 104 us, and 95 with the loads a block ahead (80 registers).
+// are formed on the FP64 and the integer pipes together (fixed.cuh): the FP64
+// pipe alone bounds the 64^3 operator (7.19 M blocks) at 107 us, HBM at 81.
+// Measured there: y = A x 128 us on the FP64 pipe alone, 95 to 98 on both with
+// the loads a block ahead (20 to 24 warps per SM).
 template <int BR, int BC, typename TM, typename TX>
 constexpr bool fx_product() {
   return BR == 3 && (BC == 3 || BC == 6) && std::is_same<TM, double>::value && std::is_same<TX, double>::value;
@@ -67,7 +68,7 @@ template <int BR, int BC, int V>
 __device__ __forceinline__ void row_sums_fx(int c0, int c1, const int* __restrict__ col,
                                             const double* __restrict__ vals, const double* __restrict__ x, int lane,
                                             double (&acc)[BR]) {
-  FxSum<BR, BC> sum;
+  FxSum<BR, BC, fx_fma_products<BR, BC>(V)> sum;
   sum.init();
   double blk[BR * BC], xv[BC];
   auto load = [&](int c, int j) {
@@ -94,13 +95,13 @@ __device__ __forceinline__ void row_sums_fx(int c0, int c1, const int* __restric
         load(c + V, next);
         if (c + 2 * V < c1) next = __ldcs(col + (int64_t)(c + 2 * V) * 32 + lane);
       }
-      sum.add(b, xb);
+      sum.add([&](int r, int q) { return b[r * BC + q]; }, xb);
     }
   } else {
 #pragma unroll 1
     for (int c = c0; c < c1; c += V) {
       load(c, __ldcs(col + (int64_t)c * 32 + lane));
-      sum.add(blk, xv);
+      sum.add([&](int r, int q) { return blk[r * BC + q]; }, xv);
     }
   }
   if (!sum.finish(acc)) row_sums<BR, BC, V, double, double, double>(c0, c1, col, vals, x, lane, acc);
@@ -420,13 +421,13 @@ __device__ __forceinline__ void row_sums4(int a0, int a1, const int* __restrict_
 }
 
 // The four vectors share a block's limbs; per vector the sums are those of
-// row_sums_fx with one lane per row, bit for bit (65^3 nodes, 16 vectors:
-// 1,820 us on the FP64 pipe alone, 959 on both).
+// row_sums_fx with one lane per row, bit for bit.
 template <int BR, int BC>
 __device__ __forceinline__ void row_sums4_fx(int a0, int a1, const int* __restrict__ col,
                                              const double* __restrict__ vals, const double* __restrict__ X, int kp,
                                              int lane, int c0, double (&acc)[BR][4]) {
-  using Row = FxRow<BR, BC>;
+  constexpr int F0 = fx_fma_products<BR, BC>(1);
+  using Row = FxRow<BR, BC, F0>;
   Row row[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) row[e].init();
@@ -440,14 +441,15 @@ __device__ __forceinline__ void row_sums4_fx(int a0, int a1, const int* __restri
     for (int e = 0; e < BR * BC; ++e) blk[e] = __ldg(v + 32 * e);
 #pragma unroll
     for (int q = 0; q < BC; ++q) ld4(X + ((int64_t)j * BC + q) * kp + c0, xv[q]);
-    FxBlock<BR, BC> a;
-    a.cut(blk);
+    const auto entry = [&](int r, int q) { return blk[r * BC + q]; };
+    FxBlock<BR, BC, F0> a;
+    a.take(entry);
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       double x[BC];
 #pragma unroll
       for (int q = 0; q < BC; ++q) x[q] = xv[q][e];
-      row[e].add(blk, a, x);
+      row[e].add(entry, a, x);
     }
     if (--left == 0) {
       left = Row::kCarry;

@@ -181,7 +181,7 @@ struct bamg_ptap {
   double* Pblk = nullptr;
   float* Pblk32 = nullptr;
   // blocks cut for the FP64 stages (fixed.cuh): A's by slot, cut for every
-  // product, and P's transposed, with the state-gated cache
+  // product, and P's transposed, behind the state gate
   unsigned *Acut = nullptr, *Pcut = nullptr;
   float* Apad = nullptr;  // A's FP32 blocks by slot, padded to 16 bytes, for every FP32 product
   uint64_t pblk_version = ~0ull, pblk32_version = ~0ull;

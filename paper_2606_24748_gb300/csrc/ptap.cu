@@ -8,10 +8,10 @@
 // Lists are fixed by the symbolic phase, so results are deterministic and no
 // atomics are used.  The gather lists keep every FMA useful (no padding to dense
 // local blocks).  The FP64 pipe, at 2 FMA/clock/SM, would take 4.0 ms for the
-// finest level's product at 64^3; a third of the rows runs there and the rest
-// in block-scaled fixed point on the integer pipes (fixed.cuh), from operands
-// cut once per block instead of once per pair (64^3: stage 1 2.86 -> 1.70 ms
-// with the cut, stage 2 1.21 -> 0.63).  Stage 1 takes its items in runs of a
+// finest level's product at 64^3; four of nine products run there and the rest
+// in fixed point on the integer pipes (fixed.cuh), from operands cut once per
+// block instead of once per pair (64^3: stage 1 2.86 -> 1.85 ms with the cut,
+// stage 2 1.21 -> 0.70).  Stage 1 takes its items in runs of a
 // row, so that a warp's lane groups share the row's A blocks; stage 2 in
 // windows ordered by work, a long list shared by up to eight warps.
 #include <algorithm>
@@ -126,28 +126,53 @@ __device__ __forceinline__ void stage2_column(int s0, int s1, const int* __restr
   }
 }
 
+// Products of a block that the FP64 stages leave on the FP64 pipe (fixed.cuh):
+// four of nine from 3-row blocks (64^3, four, five, six of nine: stage 1 with the
+// cut 1.85, 2.01, 2.29 ms, stage 2 0.70, 0.72, 0.85), five of nine for 6x6 blocks,
+// whose stage 1 with four takes 152 registers and leaves one CTA per SM.
+constexpr int stage1_fma(int bs) { return bs * bs * (bs == 3 ? 4 : 5) / 9; }
+constexpr int stage2_fma(int bs, int bsp) { return bs * bsp * (bs == 3 ? 4 : 5) / 9; }
+// CTAs of 256 threads per SM that the FP64 stages of 3-row blocks are held to:
+// 64 and 80 registers, where the compiler would take 74 and 96 and leave 24 and
+// 16 warps per SM to cover the lists' chains of loads.
+template <int BS, typename T>
+constexpr int kStage1Ctas = BS == 3 && sizeof(T) == 8 ? 4 : 0;
+template <int BS, typename T>
+constexpr int kStage2Ctas = BS == 3 && sizeof(T) == 8 ? 3 : 0;
+template <int BS>
+using ACut = FxCut<BS, BS, stage1_fma(BS)>;
+template <int BS, int BSP>
+using PCut = FxCut<BSP, BS, stage2_fma(BS, BSP)>;  // of the transposed block
+
 // The same columns with FP64 products on both pipes (fixed.cuh); false where
 // the values are not covered and the forms above have to be taken.  The six
 // lanes of an output block share A_ik (stage 1) and P_iI (stage 2), so these
 // are read cut, from block-ordered copies: a lane that cut A_ik itself read it
-// as nine sectors of the sliced storage and repeated the others' work.
+// as nine sectors of the sliced storage and repeated the others' work.  The
+// next pair's numbers are requested before this one's products.
 template <int BS, int BSP>
 __device__ __forceinline__ bool stage1_column_fx(int s0, int s1, const int* __restrict__ ea,
                                                  const int* __restrict__ ep, const uint4* __restrict__ Acut,
                                                  const double* __restrict__ Pblk, int c, double (&acc)[BS]) {
-  using Cut = FxCut<BS, BS>;
-  FxSum<BS, BS> sum;
+  using Cut = ACut<BS>;
+  constexpr int F0 = stage1_fma(BS);
+  FxSum<BS, BS, F0> sum;
   sum.init();
+  int ia = s0 < s1 ? __ldg(ea + s0) : 0, ib = s0 < s1 ? __ldg(ep + s0) : 0;
 #pragma unroll 1
   for (int s = s0; s < s1; ++s) {
-    const int64_t aslot = __ldg(ea + s);
-    const int64_t pb = __ldg(ep + s);
-    double f[Cut::F], p[BS];
+    const uint4* pa = Acut + (int64_t)ia * Cut::kWords;
+    const double* pp = Pblk + (int64_t)ib * (BS * BSP) + c;
+    if (s + 1 < s1) {
+      ia = __ldg(ea + s + 1);
+      ib = __ldg(ep + s + 1);
+    }
+    double f[F0], p[BS];
     typename Cut::Block a;
-    Cut::load(Acut + aslot * Cut::kWords, f, a);
+    Cut::load(pa, f, a);
 #pragma unroll
-    for (int q = 0; q < BS; ++q) p[q] = __ldg(Pblk + pb * (BS * BSP) + q * BSP + c);
-    sum.add(f, a, p);
+    for (int q = 0; q < BS; ++q) p[q] = __ldg(pp + q * BSP);
+    sum.add([&](int r, int q) { return f[r * BS + q]; }, a, p);
   }
   return sum.finish(acc);
 }
@@ -156,26 +181,32 @@ template <int BS, int BSP>
 __device__ __forceinline__ bool stage2_column_fx(int s0, int s1, const int* __restrict__ ep,
                                                  const int* __restrict__ ez, const uint4* __restrict__ Pcut,
                                                  const double* __restrict__ Z, int c, double (&acc)[BSP]) {
-  using Cut = FxCut<BSP, BS>;
-  FxSum<BSP, BS> sum;
+  using Cut = PCut<BS, BSP>;
+  constexpr int F0 = stage2_fma(BS, BSP);
+  FxSum<BSP, BS, F0> sum;
   sum.init();
+  int ib = s0 < s1 ? __ldg(ep + s0) : 0, iz = s0 < s1 ? __ldg(ez + s0) : 0;
 #pragma unroll 1
   for (int s = s0; s < s1; ++s) {
-    const int64_t pb = __ldg(ep + s);
-    const int64_t z = __ldg(ez + s);
-    double f[Cut::F], zc[BS];
+    const uint4* pp = Pcut + (int64_t)ib * Cut::kWords;
+    const double* pz = Z + (int64_t)iz * (BS * BSP) + c;
+    if (s + 1 < s1) {
+      ib = __ldg(ep + s + 1);
+      iz = __ldg(ez + s + 1);
+    }
+    double f[F0], zc[BS];
     typename Cut::Block p;
-    Cut::load(Pcut + pb * Cut::kWords, f, p);
+    Cut::load(pp, f, p);
 #pragma unroll
-    for (int r = 0; r < BS; ++r) zc[r] = __ldg(Z + z * (BS * BSP) + r * BSP + c);
-    sum.add(f, p, zc);
+    for (int r = 0; r < BS; ++r) zc[r] = __ldg(pz + r * BSP);
+    sum.add([&](int u, int r) { return f[u * BS + r]; }, p, zc);
   }
   return sum.finish(acc);
 }
 
 // Cut copies: A's blocks by storage slot, and P's blocks transposed, in block
 // order.  A lane packs a block; the warp writes its 32 blocks as one run.
-template <int BR, int BC, int W>
+template <int W>
 __device__ __forceinline__ void write_cut(const uint4 (&w)[W], int64_t first, int64_t n, uint4* stage,
                                           uint4* __restrict__ out) {
   const int lane = threadIdx.x & 31;
@@ -188,7 +219,7 @@ __device__ __forceinline__ void write_cut(const uint4 (&w)[W], int64_t first, in
 template <int BS>
 __global__ void __launch_bounds__(64) k_cut_slots(int64_t nslots, const double* __restrict__ vals,
                                                   uint4* __restrict__ out) {
-  using Cut = FxCut<BS, BS>;
+  using Cut = ACut<BS>;
   __shared__ uint4 stage[2][32 * Cut::kWords];
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nslots) return;  // whole warps
@@ -196,8 +227,8 @@ __global__ void __launch_bounds__(64) k_cut_slots(int64_t nslots, const double* 
 #pragma unroll
   for (int e = 0; e < BS * BS; ++e) v[e] = __ldcs(vals + vidx<BS * BS>(t, e));
   uint4 w[Cut::kWords];
-  Cut::pack(v, w);
-  write_cut<BS, BS, Cut::kWords>(w, t & ~31LL, nslots, stage[threadIdx.x >> 5], out);
+  Cut::pack([&](int r, int q) { return v[r * BS + q]; }, w);
+  write_cut<Cut::kWords>(w, t & ~31LL, nslots, stage[threadIdx.x >> 5], out);
 }
 
 // FP32 blocks by storage slot, padded (block_pitch).
@@ -232,7 +263,7 @@ __global__ void k_pad_blocks(int64_t nblk, int n, int pitch, const double* __res
 template <int BS, int BSP>
 __global__ void __launch_bounds__(64) k_cut_transposed(int64_t nblk, const double* __restrict__ Pblk,
                                                        uint4* __restrict__ out) {
-  using Cut = FxCut<BSP, BS>;
+  using Cut = PCut<BS, BSP>;
   __shared__ uint4 stage[2][32 * Cut::kWords];
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t first = t & ~31LL;
@@ -244,12 +275,12 @@ __global__ void __launch_bounds__(64) k_cut_transposed(int64_t nblk, const doubl
 #pragma unroll
     for (int u = 0; u < BSP; ++u) v[u * BS + r] = __ldg(Pblk + b * (BS * BSP) + r * BSP + u);
   uint4 w[Cut::kWords];
-  Cut::pack(v, w);
-  write_cut<BSP, BS, Cut::kWords>(w, first, nblk, stage[threadIdx.x >> 5], out);
+  Cut::pack([&](int u, int r) { return v[u * BS + r]; }, w);
+  write_cut<Cut::kWords>(w, first, nblk, stage[threadIdx.x >> 5], out);
 }
 
 template <int BS, int BSP, typename T>
-__global__ void __launch_bounds__(256) k_ptap_stage1(int64_t n1, int rounds, const int* __restrict__ item_z,
+__global__ void __launch_bounds__(256, kStage1Ctas<BS, T>) k_ptap_stage1(int64_t n1, int rounds, const int* __restrict__ item_z,
                                                      const int* __restrict__ off, const int* __restrict__ ea,
                                                      const int* __restrict__ ep, const T* __restrict__ Avals,
                                                      const T* __restrict__ Pblk, const uint4* __restrict__ Acut,
@@ -279,7 +310,7 @@ __global__ void __launch_bounds__(256) k_ptap_stage1(int64_t n1, int rounds, con
 // S warps share an item's list, each taking a run of it; their sums meet in
 // shared memory and are added in list order (S = 1: no sharing).
 template <int BS, int BSP, int S, typename T>
-__global__ void __launch_bounds__(256) k_ptap_stage2(int64_t n2, const int* __restrict__ item_slot,
+__global__ void __launch_bounds__(256, kStage2Ctas<BS, T>) k_ptap_stage2(int64_t n2, const int* __restrict__ item_slot,
                                                      const int* __restrict__ item_tslot,
                                                      const int* __restrict__ off, const int* __restrict__ ep,
                                                      const int* __restrict__ ez, const T* __restrict__ Pblk,
@@ -659,6 +690,25 @@ static Status run_stages(bamg_ptap* pl, const T* Avals, const T* Pblk, T* Z, T* 
   return Status{};
 }
 
+// Cut copy of P's blocks for the FP64 second stage.
+static Status refresh_pcut(bamg_ptap* pl, const bamg_bsr* P) {
+  cudaStream_t st = pl->ctx->stream;
+  if (!pl->Ac || P->nnzb == 0) return Status{};
+  const int words = pl->bs == 6 ? PCut<6, 6>::kWords : pl->bsp == 6 ? PCut<3, 6>::kWords : PCut<3, 3>::kWords;
+  if (!pl->Pcut) BAMG_TRY(dalloc(&pl->Pcut, P->nnzb * words * 4, st));
+  const unsigned b = (unsigned)((P->nnzb + 63) / 64);
+  uint4* out = (uint4*)pl->Pcut;
+  if (pl->bs == 6)
+    k_cut_transposed<6, 6><<<b, 64, 0, st>>>(P->nnzb, pl->Pblk, out);
+  else if (pl->bsp == 6)
+    k_cut_transposed<3, 6><<<b, 64, 0, st>>>(P->nnzb, pl->Pblk, out);
+  else
+    k_cut_transposed<3, 3><<<b, 64, 0, st>>>(P->nnzb, pl->Pblk, out);
+  BAMG_COUNT_LAUNCH;
+  BAMG_CUDA(cudaGetLastError());
+  return Status{};
+}
+
 // State gate (Sec. 3.5): the block-ordered copy of P is rebuilt only when P's
 // version differs from the cached one.
 static Status refresh_pblk(bamg_ptap* pl, bamg_bsr* P, bool fp32) {
@@ -668,20 +718,7 @@ static Status refresh_pblk(bamg_ptap* pl, bamg_bsr* P, bool fp32) {
     if (P->vals64_stale) return make_status(BAMG_ERR_STATE, "P holds only FP32 values");
     if (!pl->Pblk) BAMG_TRY(dalloc(&pl->Pblk, ne, st));
     BAMG_TRY(launch_gather_blocks(P, P->vals, pl->Pblk, st));
-    if (pl->Ac && P->nnzb > 0) {  // the second stage's cut copy
-      const int words = pl->bs == 6 ? FxCut<6, 6>::kWords : pl->bsp == 6 ? FxCut<6, 3>::kWords : FxCut<3, 3>::kWords;
-      if (!pl->Pcut) BAMG_TRY(dalloc(&pl->Pcut, P->nnzb * words * 4, st));
-      const unsigned b = (unsigned)((P->nnzb + 63) / 64);
-      uint4* out = (uint4*)pl->Pcut;
-      if (pl->bs == 6)
-        k_cut_transposed<6, 6><<<b, 64, 0, st>>>(P->nnzb, pl->Pblk, out);
-      else if (pl->bsp == 6)
-        k_cut_transposed<3, 6><<<b, 64, 0, st>>>(P->nnzb, pl->Pblk, out);
-      else
-        k_cut_transposed<3, 3><<<b, 64, 0, st>>>(P->nnzb, pl->Pblk, out);
-      BAMG_COUNT_LAUNCH;
-      BAMG_CUDA(cudaGetLastError());
-    }
+    BAMG_TRY(refresh_pcut(pl, P));
     pl->pblk_version = P->version;
     pl->pblk_refreshes++;
   }
@@ -703,7 +740,7 @@ static Status cut_operator(bamg_ptap* pl, const bamg_bsr* A) {
   cudaStream_t st = pl->ctx->stream;
   const int64_t n = A->nslots();
   if (n == 0) return Status{};
-  const int words = pl->bs == 6 ? FxCut<6, 6>::kWords : FxCut<3, 3>::kWords;
+  const int words = pl->bs == 6 ? ACut<6>::kWords : ACut<3>::kWords;
   if (!pl->Acut) BAMG_TRY(dalloc(&pl->Acut, n * words * 4, st));
   const unsigned b = (unsigned)((n + 63) / 64);
   const int pm = prof_begin(pl->ctx, pl->prof_stage1, st, 0);
