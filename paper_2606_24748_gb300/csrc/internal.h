@@ -184,7 +184,7 @@ struct bamg_ptap {
   // product, and P's transposed, behind the state gate
   unsigned *Acut = nullptr, *Pcut = nullptr;
   float* Apad = nullptr;  // A's FP32 blocks by slot, padded to 16 bytes, for every FP32 product
-  uint64_t pblk_version = ~0ull, pblk32_version = ~0ull;
+  uint64_t pblk_version = ~0ull, pblk32_version = ~0ull, pcut_version = ~0ull;
   uint64_t pblk_refreshes = 0;
   int prof_stage1 = -1, prof_stage2 = -1;  // profiling slots of the two stages (-1: none)
 };
@@ -405,6 +405,7 @@ void bsr_release(bamg_bsr* A);
 Status ptap_build(bamg_bsr* A, bamg_bsr* P, bool want_ac, bamg_ptap** plan, bamg_bsr** Ac);
 Status ptap_run(bamg_ptap* plan, bamg_bsr* A, bamg_bsr* P, bamg_bsr* Ac, bamg_prec prec, bool stage2);
 void ptap_release(bamg_ptap* plan);
+void ptap_trim(bamg_ptap* plan);  // frees what only FP64 products use; the next one rebuilds it
 // Copy sliced values to block (pattern) order.
 Status launch_gather_blocks(const bamg_bsr* A, const double* vals, double* out, cudaStream_t st);
 

@@ -879,7 +879,7 @@ static Status mg_setup_impl(bamg_mg* mg, bamg_bsr* A, const double* coords, cons
 static void trim_plans(bamg_mg* mg) {
   if (mg->opts.precision != BAMG_FP32) return;
   for (auto& L : mg->levels)
-    if (L.plan) dfree(L.plan->Acut, mg->ctx->stream);
+    if (L.plan) ptap_trim(L.plan);
 }
 
 // The coarsest factorisation needs only the last Galerkin product and is a

@@ -419,9 +419,14 @@ void ptap_release(bamg_ptap* p) {
   dfree(p->Z32, st);
   dfree(p->Pblk, st);
   dfree(p->Pblk32, st);
-  dfree(p->Acut, st);
-  dfree(p->Pcut, st);
+  ptap_trim(p);
   dfree(p->Apad, st);
+}
+
+void ptap_trim(bamg_ptap* p) {
+  dfree(p->Acut, p->ctx->stream);
+  dfree(p->Pcut, p->ctx->stream);
+  p->pcut_version = ~0ull;
 }
 
 Status ptap_build(bamg_bsr* A, bamg_bsr* P, bool want_ac, bamg_ptap** plan_out, bamg_bsr** Ac_out) {
@@ -690,25 +695,6 @@ static Status run_stages(bamg_ptap* pl, const T* Avals, const T* Pblk, T* Z, T* 
   return Status{};
 }
 
-// Cut copy of P's blocks for the FP64 second stage.
-static Status refresh_pcut(bamg_ptap* pl, const bamg_bsr* P) {
-  cudaStream_t st = pl->ctx->stream;
-  if (!pl->Ac || P->nnzb == 0) return Status{};
-  const int words = pl->bs == 6 ? PCut<6, 6>::kWords : pl->bsp == 6 ? PCut<3, 6>::kWords : PCut<3, 3>::kWords;
-  if (!pl->Pcut) BAMG_TRY(dalloc(&pl->Pcut, P->nnzb * words * 4, st));
-  const unsigned b = (unsigned)((P->nnzb + 63) / 64);
-  uint4* out = (uint4*)pl->Pcut;
-  if (pl->bs == 6)
-    k_cut_transposed<6, 6><<<b, 64, 0, st>>>(P->nnzb, pl->Pblk, out);
-  else if (pl->bsp == 6)
-    k_cut_transposed<3, 6><<<b, 64, 0, st>>>(P->nnzb, pl->Pblk, out);
-  else
-    k_cut_transposed<3, 3><<<b, 64, 0, st>>>(P->nnzb, pl->Pblk, out);
-  BAMG_COUNT_LAUNCH;
-  BAMG_CUDA(cudaGetLastError());
-  return Status{};
-}
-
 // State gate (Sec. 3.5): the block-ordered copy of P is rebuilt only when P's
 // version differs from the cached one.
 static Status refresh_pblk(bamg_ptap* pl, bamg_bsr* P, bool fp32) {
@@ -718,7 +704,6 @@ static Status refresh_pblk(bamg_ptap* pl, bamg_bsr* P, bool fp32) {
     if (P->vals64_stale) return make_status(BAMG_ERR_STATE, "P holds only FP32 values");
     if (!pl->Pblk) BAMG_TRY(dalloc(&pl->Pblk, ne, st));
     BAMG_TRY(launch_gather_blocks(P, P->vals, pl->Pblk, st));
-    BAMG_TRY(refresh_pcut(pl, P));
     pl->pblk_version = P->version;
     pl->pblk_refreshes++;
   }
@@ -732,6 +717,26 @@ static Status refresh_pblk(bamg_ptap* pl, bamg_bsr* P, bool fp32) {
     }
     pl->pblk32_version = P->version;
   }
+  return Status{};
+}
+
+// Cut copy of P's blocks for the FP64 second stage, behind the same state gate.
+static Status refresh_pcut(bamg_ptap* pl, const bamg_bsr* P) {
+  cudaStream_t st = pl->ctx->stream;
+  if (pl->pcut_version == P->version || P->nnzb == 0) return Status{};
+  const int words = pl->bs == 6 ? PCut<6, 6>::kWords : pl->bsp == 6 ? PCut<3, 6>::kWords : PCut<3, 3>::kWords;
+  if (!pl->Pcut) BAMG_TRY(dalloc(&pl->Pcut, P->nnzb * words * 4, st));
+  const unsigned b = (unsigned)((P->nnzb + 63) / 64);
+  uint4* out = (uint4*)pl->Pcut;
+  if (pl->bs == 6)
+    k_cut_transposed<6, 6><<<b, 64, 0, st>>>(P->nnzb, pl->Pblk, out);
+  else if (pl->bsp == 6)
+    k_cut_transposed<3, 6><<<b, 64, 0, st>>>(P->nnzb, pl->Pblk, out);
+  else
+    k_cut_transposed<3, 3><<<b, 64, 0, st>>>(P->nnzb, pl->Pblk, out);
+  BAMG_COUNT_LAUNCH;
+  BAMG_CUDA(cudaGetLastError());
+  pl->pcut_version = P->version;
   return Status{};
 }
 
@@ -780,13 +785,14 @@ Status ptap_run(bamg_ptap* pl, bamg_bsr* A, bamg_bsr* P, bamg_bsr* Ac, bamg_prec
   if (prec == BAMG_FP64) {
     if (A->vals64_stale) return make_status(BAMG_ERR_STATE, "A holds only FP32 values; use BAMG_FP32");
     BAMG_TRY(refresh_pblk(pl, P, false));
+    if (stage2) BAMG_TRY(refresh_pcut(pl, P));
     BAMG_TRY(cut_operator(pl, A));
     BAMG_TRY(run_stages<double>(pl, A->vals, pl->Pblk, pl->Z, stage2 ? Ac->vals : nullptr, stage2));
     if (stage2) {
       Ac->version++;
       Ac->vals64_stale = false;
     } else {
-      dfree(pl->Acut, st);  // prolongator smoothing: setup only
+      ptap_trim(pl);  // prolongator smoothing: setup only
     }
   } else if (prec == BAMG_FP32) {
     BAMG_TRY(bsr_ensure_fp32(A));
