@@ -335,8 +335,13 @@ __global__ void __launch_bounds__(fx_product<BS, BS, TM, double>() ? kFxRedThrea
 
 // The same step (block diagonal only) in the component-split form for 6-row
 // blocks: CTA = one slice at a time (grid-stride over slices), BS * VS warps.
+// Two and four warps per component are held to 40 registers: at the 58 that the
+// compiler takes with the cluster's sums one CTA of 768 threads fills an SM
+// (64^3, level 1, four warps: 39.6 us FP64 and 52.8 FP32, so 28.9 and 46.8; two
+// warps 40.4 and 54.6, so 30.9 and 50.9).  One warp per component has the room
+// (34.0 us, 35.4 if held).
 template <int BS, int VS, typename TM>
-__global__ void __launch_bounds__(768) k_power_step_split(const int* __restrict__ slice_ptr,
+__global__ void __launch_bounds__(768, VS == 1 ? 0 : 2) k_power_step_split(const int* __restrict__ slice_ptr,
                                                           const int* __restrict__ col, const TM* __restrict__ vals,
                                                           const int* __restrict__ srow,
                                                           const double* __restrict__ dinv,
