@@ -377,8 +377,12 @@ __global__ void __launch_bounds__(768, VS == 1 ? 0 : 2) k_power_step_split(const
 
 // Rayleigh quotient w^T A w / w^T D w; in block mode also the Chebyshev data
 // for the interval [lower, upper] * lambda (Saad, Alg. 12.1 coefficients).
+// The FP64 3x3 form is held to the six CTAs per SM of its grid (fx_red_grid): at
+// the 96 registers that the compiler takes five are resident and the sixth is a
+// second wave (64^3: 165 us, 113 held).
 template <int BS, int V, typename TM>
-__global__ void __launch_bounds__(fx_product<BS, BS, TM, double>() ? kFxRedThreads : 256) k_rayleigh(const int* __restrict__ slice_ptr,
+__global__ void __launch_bounds__(fx_product<BS, BS, TM, double>() ? kFxRedThreads : 256,
+                                  fx_product<BS, BS, TM, double>() ? 6 : 0) k_rayleigh(const int* __restrict__ slice_ptr,
                                                           const int* __restrict__ col, const TM* __restrict__ vals,
                                                           const int* __restrict__ srow,
                                                           const int* __restrict__ diag_slot, int scalar_diag,
