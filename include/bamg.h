@@ -479,8 +479,9 @@ BAMG_API bamg_status bamg_cg_solve(bamg_mg* mg, const double* b, double* x, doub
  * bamg_mg_vcycle_multi: X = M B, one V-cycle per column from x = 0.  Per
  * column the arithmetic and its order are those of bamg_vcycle with one lane
  * per block row on every operator (bamg_bsr_set_lanes(.., 1)), so the
- * results then agree bit for bit; with other lane counts they differ by
- * rounding.
+ * results then agree bit for bit.  Otherwise they differ by rounding: operators
+ * with few rows then share each row's blocks among threads, in a way that
+ * follows from their sizes and not from the lanes, tuned or set.
  *
  * bamg_cg_solve_multi: k independent preconditioned CG recurrences (the
  * iterates of bamg_cg_solve on each column, up to the summation order of the

@@ -210,6 +210,7 @@ Status bsr_set_pattern(bamg_bsr* A, std::vector<int>&& rowptr, std::vector<int>&
   A->has_pattern = true;
   A->vec = A->vec32 = default_vec(A);
   A->vec_tuned = false;
+  A->one_lane = A->one_lane32 = false;
   A->version++;
   static uint64_t next_pattern_id = 0;
   A->pattern_id = ++next_pattern_id;
@@ -519,6 +520,7 @@ bamg_status bamg_bsr_set_lanes(bamg_bsr* A, int lanes) {
   if (!s.ok()) return fail(A->ctx, s);
   if (!split) A->vec = A->vec32 = vec;
   A->split = A->split32 = split;
+  A->one_lane = A->one_lane32 = lanes == 1;
   return BAMG_OK;
 }
 
@@ -537,6 +539,7 @@ bamg_status bamg_bsr_set_lanes_prec(bamg_bsr* A, int prec, int lanes) {
   if (!s.ok()) return fail(A->ctx, s);
   if (!sp) vec = v;
   split = sp;
+  (prec == BAMG_FP64 ? A->one_lane : A->one_lane32) = lanes == 1;
   return BAMG_OK;
 }
 

@@ -134,6 +134,7 @@ struct bamg_bsr {
   int split32 = 0;           //   that many warps per component of a slice; 32, 64, 128 = one CTA per
                              //   row, split / 32 warps per component (FP64 / FP32 kernels)
   bool vec_tuned = false;
+  bool one_lane = false, one_lane32 = false;  // the caller fixed one lane per row (FP64 / FP32 kernels)
   std::vector<int> h_slice_ptr, h_slot_of;
   double* vals = nullptr;    // 32 * nchunks * B
   float* vals32 = nullptr;   // float copy in the same layout

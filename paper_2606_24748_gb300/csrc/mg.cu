@@ -1085,6 +1085,7 @@ bamg_status bamg_mg_set_lanes(bamg_mg* mg, int lanes) {
         const bool split = lanes == 0 && M->br == 6 && (M->bc == 3 || M->bc == 6);
         M->vec = M->vec32 = lanes == 0 ? 1 : lanes;
         M->split = M->split32 = split ? 4 : 0;
+        M->one_lane = M->one_lane32 = !split && M->vec == 1;
       }
   mg_release_graphs(mg);  // captured iterations hold the old launch shapes
   return BAMG_OK;

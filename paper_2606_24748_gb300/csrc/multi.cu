@@ -610,13 +610,13 @@ MPtrs<T> mptrs(Level& L, MultiLevel& W) {
 // of the FP64 pipes (1,331 rows x 16 columns, 27 6x6 blocks: 177 us unsplit,
 // 37 us split).  FP64 3x3 products also use the integer pipes (fixed.cuh)
 // and stay unsplit down to 256 warps.  A row is shared by as many threads as
-// it takes to reach four warps per sub-partition, at most one per block.  A
-// matrix set to one lane per row is never split: its columns are then summed
-// as the single-vector kernels sum them.
+// it takes to reach four warps per sub-partition, at most one per block.  The
+// choice depends on sizes alone, never on what the tuner timed for single
+// vectors, but a matrix that the caller set to one lane per row is not split:
+// its columns are then summed as the single-vector kernels sum them.
 template <typename T>
 bool split_map(const bamg_bsr* M, int kp, SplitMap& m) {
-  const int vec = sizeof(T) == 4 ? M->vec32 : M->vec, split = sizeof(T) == 4 ? M->split32 : M->split;
-  if ((vec <= 1 && split == 0) || M->nbr == 0) return false;
+  if ((sizeof(T) == 4 ? M->one_lane32 : M->one_lane) || M->nbr == 0) return false;
   const bool fx = sizeof(T) == 8 && M->br == 3 && M->bc == 3;
   if (M->nbr * kp / 128 >= (fx ? 256 : 1216)) return false;
   const int64_t blocks = std::max<int64_t>(1, M->nnzb / M->nbr);

@@ -315,8 +315,14 @@ Status bsr_autotune(bamg_bsr* A, float* best_ms) {
   if (!A->has_pattern) return make_status(BAMG_ERR_STATE, "autotune needs a pattern");
   const bool special = (A->br == 3 || A->br == 6) && (A->bc == 3 || A->bc == 6);
   if (!special) return Status{};
-  if (!A->vals64_stale) BAMG_TRY(tune_lanes<double>(A, A->vals, &A->vec, &A->split, best_ms));
-  if (A->vals32) BAMG_TRY(tune_lanes<float>(A, A->vals32, &A->vec32, &A->split32, A->vals64_stale ? best_ms : nullptr));
+  if (!A->vals64_stale) {
+    BAMG_TRY(tune_lanes<double>(A, A->vals, &A->vec, &A->split, best_ms));
+    A->one_lane = false;
+  }
+  if (A->vals32) {
+    BAMG_TRY(tune_lanes<float>(A, A->vals32, &A->vec32, &A->split32, A->vals64_stale ? best_ms : nullptr));
+    A->one_lane32 = false;
+  }
   A->vec_tuned = true;
   return Status{};
 }

@@ -229,3 +229,23 @@ def test_split_rows_give_the_unsplit_cycle(precision, tol, aggregation, ne, ks):
                 assert rel(X[:, j].cpu().numpy(), Y[:, j].cpu().numpy()) <= tol, (k, j)
     finally:
         gp.close()
+
+
+@pytest.mark.parametrize("precision", [B.BAMG_FP64, B.BAMG_FP32])
+@pytest.mark.parametrize("aggregation,ne", [(B.BAMG_AGG_GEOMETRIC, 13), (B.BAMG_AGG_MIS, 12)])
+def test_columns_do_not_depend_on_tuned_lanes(precision, aggregation, ne):
+    """The multi-vector kernels' mapping follows from sizes: the tuner's choices
+    and every lane count but one (documented to sum as the single-vector cycle
+    of one lane) give the same bits."""
+    gp = GpuProblem(ne, precision=precision, aggregation=aggregation)
+    try:
+        for k in (3, 16):
+            Bh = dev(rhs(gp.mesh, k, 60))
+            X, Y = torch.zeros_like(Bh), torch.zeros_like(Bh)
+            B.bamg_mg_vcycle_multi(gp.ctx, gp.mg, Bh, X, k)
+            for lanes in (2, 4, 32):
+                B.bamg_mg_set_lanes(gp.ctx, gp.mg, lanes)
+                B.bamg_mg_vcycle_multi(gp.ctx, gp.mg, Bh, Y, k)
+                assert torch.equal(X, Y), (k, lanes)
+    finally:
+        gp.close()
