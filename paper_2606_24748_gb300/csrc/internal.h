@@ -475,7 +475,7 @@ inline int split_for(const bamg_bsr* A) {
 // with two chunks or more per warp.
 inline int split_cluster(const bamg_bsr* A, int vs) {
   if (A->nslices <= 0) return 1;
-  const int64_t chunks = A->nchunks / A->nslices, resident = 152 * std::min(4, 2048 / (192 * vs));
+  const int64_t chunks = A->nchunks / A->nslices, resident = (int64_t)A->ctx->sm_count * std::min(4, 2048 / (192 * vs));
   int n = 1;
   while (n < 8 && A->nslices * 2 * n <= resident && chunks >= 2LL * (2 * n) * vs) n *= 2;
   return n;

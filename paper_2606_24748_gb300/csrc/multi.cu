@@ -606,23 +606,26 @@ MPtrs<T> mptrs(Level& L, MultiLevel& W) {
 
 // Whether a matrix's multi-vector kernels run in the split form, and its
 // mapping.  The unsplit form's 4-column threads fill n kp / 128 warps; below
-// two per SM sub-partition (1,216) the kernels wait on the longest row instead
-// of the FP64 pipes (1,331 rows x 16 columns, 27 6x6 blocks: 177 us unsplit,
-// 37 us split).  FP64 3x3 products also use the integer pipes (fixed.cuh)
-// and stay unsplit down to 256 warps.  A row is shared by as many threads as
-// it takes to reach four warps per sub-partition, at most one per block.  The
-// choice depends on sizes alone, never on what the tuner timed for single
-// vectors, but a matrix that the caller set to one lane per row is not split:
-// its columns are then summed as the single-vector kernels sum them.
+// two per SM sub-partition (1,216 on 152 SMs) the kernels wait on the longest
+// row instead of the FP64 pipes (1,331 rows x 16 columns, 27 6x6 blocks: 177 us
+// unsplit, 37 us split).  FP64 3x3 products also use the integer pipes
+// (fixed.cuh) and stay unsplit down to 256 warps (1.7 per SM).  A row is shared
+// by as many threads as it takes to reach four warps per sub-partition, at most
+// one per block.  The choice depends on sizes alone, never on what the tuner
+// timed for single vectors, but a matrix that the caller set to one lane per row
+// is not split: its columns are then summed as the single-vector kernels sum
+// them.
 template <typename T>
 bool split_map(const bamg_bsr* M, int kp, SplitMap& m) {
   if ((sizeof(T) == 4 ? M->one_lane32 : M->one_lane) || M->nbr == 0) return false;
   const bool fx = sizeof(T) == 8 && M->br == 3 && M->bc == 3;
-  if (M->nbr * kp / 128 >= (fx ? 256 : 1216)) return false;
+  const int64_t sms = M->ctx->sm_count;
+  if (M->nbr * kp / 128 >= (fx ? 256 * sms / 152 : 8 * sms)) return false;
   const int64_t blocks = std::max<int64_t>(1, M->nnzb / M->nbr);
   m.klog = ilog2(kp);
   m.vlog = 1;
-  while (M->nbr * kp / 32 << m.vlog < 2432 && (2 << m.vlog) <= blocks && (kp << (m.vlog + 1)) <= kSplitThreads) ++m.vlog;
+  while (M->nbr * kp / 32 << m.vlog < 16 * sms && (2 << m.vlog) <= blocks && (kp << (m.vlog + 1)) <= kSplitThreads)
+    ++m.vlog;
   m.rlog = std::max(0, 8 - m.klog - m.vlog);  // CTAs of 256 threads, 512 for kp x 2^vlog = 512
   return true;
 }

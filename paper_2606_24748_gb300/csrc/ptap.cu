@@ -368,11 +368,11 @@ __global__ void __launch_bounds__(256, kStage2Ctas<BS, T>) k_ptap_stage2(int64_t
 // share operand blocks (one row's and its neighbours') meet in one L1 while the
 // lane groups of a warp still carry equal work; sorted over all items, every
 // block comes from L2 or HBM once per list it is in (64^3: 2.27 -> 1.93 ms).
-// More rounds share more but leave fewer CTAs: eight where each of 152 SMs
-// still gets eight CTAs.  Stage 2's lists differ too much in length within a
+// More rounds share more but leave fewer CTAs: eight where each SM still gets
+// eight CTAs.  Stage 2's lists differ too much in length within a
 // run (0.63 ms sorted over all items, 1.07 in runs).
-static int item_rounds(int64_t items, int bsp) {
-  return (int)std::max<int64_t>(1, std::min<int64_t>(8, items / (8 * (32 / bsp) * 152 * 8)));
+static int item_rounds(int64_t items, int bsp, int sm_count) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(8, items / (8 * (32 / bsp) * sm_count * 8)));
 }
 
 // Stable order of items by decreasing list length within runs of `window`.
@@ -510,7 +510,7 @@ Status ptap_build(bamg_bsr* A, bamg_bsr* P, bool want_ac, bamg_ptap** plan_out, 
     pl->n1 = pl->nz;
     pl->e1 = (int64_t)la.size();
     {
-      pl->rounds1 = item_rounds(pl->n1, bsp);
+      pl->rounds1 = item_rounds(pl->n1, bsp, pl->ctx->sm_count);
       std::vector<int> order = order_by_work(off1, pl->rounds1 * 8 * (32 / bsp)), noff, na, np;
       permute_lists(order, off1, la, lp, noff, na, np);
       BAMG_TRY(upload(&pl->s1_z, order, st));
@@ -665,7 +665,7 @@ static Status run_stages(bamg_ptap* pl, const T* Avals, const T* Pblk, T* Z, T* 
     // them until there are 16 per SM sub-partition (64^3, level 1: 3,601 items
     // are 91 CTAs and took 321 us; 12^3, level 0: 125 -> 23 us shared by eight).
     int S = 1;
-    while (S < 8 && pl->n2 / G * S < 152 * 4 * 16) S *= 2;
+    while (S < 8 && pl->n2 / G * S < pl->ctx->sm_count * 4 * 16) S *= 2;
     const int64_t per = (int64_t)(8 / S) * G;
     const unsigned b = (unsigned)((pl->n2 + per - 1) / per);
     const int pm = prof_begin(pl->ctx, pl->prof_stage2, st);
