@@ -40,8 +40,8 @@ METRIC = "PtAP+V-cycle HBM GB/s; CG time to rtol 1e-8, FP64 vs mixed/learned"
 # FP64 FMA peak from unit counts and the maximum clock: SMs x DFMA/clk/SM x
 # flop/FMA x 2.07 GHz.  The roofline's denominator for FP64-bound kernels.  A
 # pure-FMA probe (bamg_probe_fma_rate) is measured beside it and stays below
-# this figure.  The 3x3 products run three or four of nine multiply-adds on the
-# integer pipes (csrc/fixed.cuh) and can pass it.
+# this figure.  Of the 3x3 products' nine multiply-adds per block three or four
+# run on the integer pipes (csrc/fixed.cuh) and are not counted against it.
 FP64_PEAK_DERIVED_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
 RTOL = 1e-8
 MAXIT = 500
@@ -509,7 +509,8 @@ def roofline(wl, prof, B, alu):
     s = 4 if wl.mixed else 8
     n, nnzb = A0["nbr"], A0["nnzb"]
     cand = {}
-    fl = 2 * nnzb * 9 + n * (2 * 9 + 8)
+    # of nine multiply-adds per block at most six run on the FP64 pipe (csrc/fixed.cuh)
+    fl = 2 * nnzb * 6 + n * (2 * 9 + 8)
     if prof.get("cheb_pre_l0", (0, 0))[1]:
         # the sampled pre-smoothing pair: step 0 with a next direction, then the last pre step
         bts = (bm.cheb_step_bytes(nnzb, n, 3, s, True) + bm.cheb_step_bytes(nnzb, n, 3, s, False)) / 2
@@ -525,7 +526,7 @@ def roofline(wl, prof, B, alu):
                            None)
     if prof["cg_ap"][1]:
         bts = bm.spmv_bytes(nnzb, n, n, 3, 3, 8) + 8 * 3 * n
-        cand["cg_ap"] = (prof["cg_ap"], bts, 2 * nnzb * 9 + 6 * n)
+        cand["cg_ap"] = (prof["cg_ap"], bts, 2 * nnzb * 6 + 6 * n)
     if not cand:
         return None
     name = max(cand, key=lambda k: cand[k][0][0])
@@ -546,9 +547,9 @@ def roofline(wl, prof, B, alu):
         tf = fl / avg_s / 1e12
         out.update({"bound": "alu", "achieved": round(tf, 4), "peak": peak64,
                     "unit": "TFLOP/s", "frac": round(tf / peak64, 3),
-                    "peak_source": "FP64 FMA pipe alone, from unit counts and the maximum clock (152 x 2 DFMA/clk x "
-                                   "2 flop x 2.07 GHz); three or four of a block's nine products run on the "
-                                   "integer pipes, so the fraction may exceed 1 (hbm_frac is the other bound)",
+                    "peak_source": "FP64 FMA pipe, from unit counts and the maximum clock (152 x 2 DFMA/clk x "
+                                   "2 flop x 2.07 GHz); without the three of a block's nine products that run on "
+                                   "the integer pipes",
                     "probe_tflops": alu["fp64_probe_tflops"]})
     else:
         out.update({"bound": "hbm", "achieved": round(gbs, 1), "peak": hbm, "unit": "GB/s",
