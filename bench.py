@@ -40,7 +40,7 @@ METRIC = "PtAP+V-cycle HBM GB/s; CG time to rtol 1e-8, FP64 vs mixed/learned"
 # FP64 FMA peak from unit counts and the maximum clock: SMs x DFMA/clk/SM x
 # flop/FMA x 2.07 GHz.  The roofline's denominator for FP64-bound kernels.  A
 # pure-FMA probe (bamg_probe_fma_rate) is measured beside it and stays below
-# this figure.  Of the 3x3 products' nine multiply-adds per block three or four
+# this figure.  Of the 3x3 products' nine multiply-adds per block three or five
 # run on the integer pipes (csrc/fixed.cuh) and are not counted against it.
 FP64_PEAK_DERIVED_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
 RTOL = 1e-8
@@ -52,8 +52,8 @@ MAXIT = 500
 # null once it changes.  The source is device.cuh (the row products),
 # fixed.cuh (their fixed-point part) and the span of cycle.cu from the
 # block-diagonal apply through the end of the fused Chebyshev step.
-TRAFFIC = {("cheb_step_l0", 64, False): (586.7e6, "c7fdfebe78bc399f"),
-           ("cheb_step_l0", 64, True): (307.7e6, "c7fdfebe78bc399f")}
+TRAFFIC = {("cheb_step_l0", 64, False): (587.0e6, "741c46102c92c526"),
+           ("cheb_step_l0", 64, True): (307.7e6, "741c46102c92c526")}
 TRAFFIC_SOURCES = (("paper_2606_24748_gb300/csrc/device.cuh", None, None),
                    ("paper_2606_24748_gb300/csrc/fixed.cuh", None, None),
                    ("paper_2606_24748_gb300/csrc/cycle.cu", "__device__ __forceinline__ void dinv_apply",
@@ -549,7 +549,7 @@ def roofline(wl, prof, B, alu):
                     "unit": "TFLOP/s", "frac": round(tf / peak64, 3),
                     "peak_source": "FP64 FMA pipe, from unit counts and the maximum clock (152 x 2 DFMA/clk x "
                                    "2 flop x 2.07 GHz); without the three of a block's nine products that run on "
-                                   "the integer pipes",
+                                   "the integer pipes at the least",
                     "probe_tflops": alu["fp64_probe_tflops"]})
     else:
         out.update({"bound": "hbm", "achieved": round(gbs, 1), "peak": hbm, "unit": "GB/s",

@@ -37,8 +37,8 @@ __device__ __forceinline__ double warp_sum(double v) {
 // FP64 products of 3x3 and 3x6 blocks (the finest operator and prolongator)
 // are formed on the FP64 and the integer pipes together (fixed.cuh): the FP64
 // pipe alone bounds the 64^3 operator (7.19 M blocks) at 107 us, HBM at 81.
-// Measured there: y = A x 128 us on the FP64 pipe alone, 95 to 98 on both with
-// the loads a block ahead (20 to 24 warps per SM).
+// Measured there: y = A x 128 us on the FP64 pipe alone, 96 on both with the
+// loads a block ahead.
 template <int BR, int BC, typename TM, typename TX>
 constexpr bool fx_product() {
   return BR == 3 && (BC == 3 || BC == 6) && std::is_same<TM, double>::value && std::is_same<TX, double>::value;

@@ -21,8 +21,8 @@
 // off by n 2^-53 of the sum of |a| |x|, which is no less, so values of unlike
 // size in a block or in x cost no more bits here than there.  Measured against
 // 113-bit sums, root mean square of error over sum of |a| |x|, rows of 1 to 90
-// 3x3 blocks: 3.7e-17 here (four of nine products in fixed point) and 5.2e-17
-// by FP64 FMA; with rows, columns or entries over 24 decades 3.9e-17 to 1.7e-16
+// 3x3 blocks: 3.3e-17 here (five of nine products in fixed point) and 5.2e-17
+// by FP64 FMA; with rows, columns or entries over 24 decades 3.5e-17 to 1.5e-16
 // and 5.2e-17 to 2.1e-16.  (One scale for the rows of a block, and one for x's
 // entries, would take fewer operations, but lose the small rows and entries of a
 // block beside large ones.)  Cuts are symmetric in the sign and move with the
@@ -36,15 +36,15 @@
 namespace bamg {
 
 // Products of a block (row-major) that stay on the FP64 pipe; the last row of
-// these may be divided.  Five of nine with one lane per row (64^3, y = A x with
-// four, five, six: 95, 94, 92 us, but the fused Chebyshev step 105, 105, 111 and
-// the CG product 133, 111, 113; 16 vectors at 48^3 498, 501, 522): with six the
-// FP64 pipe is 0.91 busy where products follow one another.  Six of nine for
-// several lanes per row, which have few blocks each, so that only one of three
-// rows has fixed-point sums to shift and convert (24^3, fine Chebyshev step 16.7
-// us, 19.2 with five).
+// these may be divided.  Four of nine with one lane per row: at 64^3 with three,
+// four, five, six of nine y = A x takes 95, 96, 98, 99 us, the fused Chebyshev
+// step 108, 106, 106, 110 and the CG product 133 (spills), 109, 107, 109; 16
+// vectors at 48^3 442, 447, 474, 518.  With six the FP64 pipe is 0.91 busy where
+// products follow one another.  Six of nine for several lanes per row, which have
+// few blocks each, so that only one of three rows has fixed-point sums to shift
+// and convert (24^3, fine Chebyshev step 16.7 us, 19.2 with five).
 template <int BR, int BC>
-constexpr int fx_fma_products(int lanes) { return BR * BC * (lanes == 1 ? 5 : 6) / 9; }
+constexpr int fx_fma_products(int lanes) { return BR * BC * (lanes == 1 ? 4 : 6) / 9; }
 
 // Exponents are biased, less one.  A zero's is so far below all others that a
 // product with it is shifted out at every scale and does not raise one (kFxNone:
