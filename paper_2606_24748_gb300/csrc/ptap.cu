@@ -128,17 +128,20 @@ __device__ __forceinline__ void stage2_column(int s0, int s1, const int* __restr
 
 // Products of a block that the FP64 stages leave on the FP64 pipe (fixed.cuh):
 // four of nine from 3-row blocks (64^3, four, five, six of nine: stage 1 with the
-// cut 1.85, 2.01, 2.29 ms, stage 2 0.70, 0.72, 0.85), five of nine for 6x6 blocks,
-// whose stage 1 with four takes 152 registers and leaves one CTA per SM.
-constexpr int stage1_fma(int bs) { return bs * bs * (bs == 3 ? 4 : 5) / 9; }
-constexpr int stage2_fma(int bs, int bsp) { return bs * bsp * (bs == 3 ? 4 : 5) / 9; }
-// CTAs of 256 threads per SM that the FP64 stages of 3-row blocks are held to:
-// 64 and 80 registers, where the compiler would take 74 and 96 and leave 24 and
-// 16 warps per SM to cover the lists' chains of loads.
+// cut 1.85, 2.01, 2.29 ms, stage 2 0.70, 0.72, 0.85), three of nine for 6x6
+// blocks (MIS hierarchy at 48^3, both its products, two, three, four, five, six:
+// stage 1 4.95, 4.01, 4.24, 4.61, 5.20 ms; stage 2 1.25, 1.34, 1.53, 1.75 with
+// three to six).
+constexpr int stage1_fma(int bs) { return bs * bs * (bs == 3 ? 4 : 3) / 9; }
+constexpr int stage2_fma(int bs, int bsp) { return bs * bsp * (bs == 3 ? 4 : 3) / 9; }
+// CTAs of 256 threads per SM that the FP64 stages are held to.  3-row blocks: 64
+// and 80 registers, where the compiler would take 74 and 96 and leave 24 and 16
+// warps per SM to cover the lists' chains of loads; 6x6: 128, where it would take
+// 152 and leave one CTA (stage 2 of the 48^3 example 1.97 ms so).
 template <int BS, typename T>
-constexpr int kStage1Ctas = BS == 3 && sizeof(T) == 8 ? 4 : 0;
+constexpr int kStage1Ctas = sizeof(T) == 8 ? (BS == 3 ? 4 : 2) : 0;
 template <int BS, typename T>
-constexpr int kStage2Ctas = BS == 3 && sizeof(T) == 8 ? 3 : 0;
+constexpr int kStage2Ctas = sizeof(T) == 8 ? (BS == 3 ? 3 : 2) : 0;
 template <int BS>
 using ACut = FxCut<BS, BS, stage1_fma(BS)>;
 template <int BS, int BSP>
