@@ -52,8 +52,8 @@ MAXIT = 500
 # null once it changes.  The source is device.cuh (the row products),
 # fixed.cuh (their fixed-point part) and the span of cycle.cu from the
 # block-diagonal apply through the end of the fused Chebyshev step.
-TRAFFIC = {("cheb_step_l0", 64, False): (587.0e6, "741c46102c92c526"),
-           ("cheb_step_l0", 64, True): (307.7e6, "741c46102c92c526")}
+TRAFFIC = {("cheb_step_l0", 64, False): (588.2e6, "b7a359e5c769a884"),
+           ("cheb_step_l0", 64, True): (307.6e6, "b7a359e5c769a884")}
 TRAFFIC_SOURCES = (("paper_2606_24748_gb300/csrc/device.cuh", None, None),
                    ("paper_2606_24748_gb300/csrc/fixed.cuh", None, None),
                    ("paper_2606_24748_gb300/csrc/cycle.cu", "__device__ __forceinline__ void dinv_apply",

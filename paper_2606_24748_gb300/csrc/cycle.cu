@@ -63,13 +63,28 @@ __global__ void __launch_bounds__(kRowThreads) k_cheb_init(int64_t n, const TB* 
   }
 }
 
+// CTA size of the fused Chebyshev row kernels.  A level's rows fill about one
+// wave of the GPU at the workload sizes (64^3: 8,582 slices for 152 SMs x 64
+// warps), so the last CTA of the busier SMs is the kernel's tail: 64-thread
+// CTAs (two slices) halve it against 128-thread ones.
+constexpr int kChebThreads = 64;
+// The FP64 3x3 forms are held to eleven of them on an SM (88 registers): at the
+// 86 to 94 that the compiler takes, ten or eleven, and a count of CTAs near a
+// whole wave then makes one more (59^3, fused step: 92 us free, 82 held; with
+// twelve 83).
+template <int BS, typename T>
+constexpr int kChebCtas = fx_product<BS, BS, T, T>() ? 11 : 0;
+template <int BS, typename T>
+constexpr int kChebBound = fx_product<BS, BS, T, T>() ? kChebThreads : kRowThreads;
+
 // x += d_in; r -= A d_in; if has_next: d_out = c1 d_in + c2 w Dinv r.
 // FINAL (the last step of post-smoothing): the next direction is the last
 // one; it is added to x here ((x + d_in) + d_out, the order of a separate
 // update) instead of being stored.  A separate instance, so that the common
 // one keeps its register count.
 template <int BS, int V, typename T, bool FINAL = false>
-__global__ void __launch_bounds__(kRowThreads) k_cheb_step(const int* __restrict__ sp, const int* __restrict__ col,
+__global__ void __launch_bounds__(kChebBound<BS, T>, kChebCtas<BS, T>)
+    k_cheb_step(const int* __restrict__ sp, const int* __restrict__ col,
                                                            const T* __restrict__ vals, const int* __restrict__ srow,
                                                            int64_t n, int64_t nthreads,
                                                            const T* __restrict__ d_in, T* __restrict__ d_out,
@@ -119,7 +134,8 @@ __global__ void __launch_bounds__(kRowThreads) k_cheb_step(const int* __restrict
 
 // r = b - A x; d = w Dinv r / theta   (x is read by the product: not written here)
 template <int BS, int V, typename T>
-__global__ void __launch_bounds__(kRowThreads) k_cheb_rinit(const int* __restrict__ sp, const int* __restrict__ col,
+__global__ void __launch_bounds__(kChebBound<BS, T>, kChebCtas<BS, T>)
+    k_cheb_rinit(const int* __restrict__ sp, const int* __restrict__ col,
                                                             const T* __restrict__ vals, const int* __restrict__ srow,
                                                             int64_t n, int64_t nthreads,
                                                             const T* __restrict__ x, const T* __restrict__ b,
@@ -337,12 +353,6 @@ template <>
 LevelPtrs<double> level_ptrs<double>(Level& L) { return ptrs64(L); }
 template <>
 LevelPtrs<float> level_ptrs<float>(Level& L) { return ptrs32(L); }
-
-// CTA size of the fused Chebyshev row kernels.  A level's rows fill about one
-// wave of the GPU at the workload sizes (64^3: 8,582 slices for 152 SMs x 64
-// warps), so the last CTA of the busier SMs is the kernel's tail: 64-thread
-// CTAs (two slices) halve it against 128-thread ones.
-constexpr int kChebThreads = 64;
 
 // b64 (mixed form, finest level): the FP64 right-hand side, converted by the
 // first kernel; p.b then receives its float copy.
